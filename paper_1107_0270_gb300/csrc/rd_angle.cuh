@@ -33,41 +33,30 @@
 namespace rd {
 
 constexpr int kAngNMax = 128;          // partial waves at most (kappa = R' R0 / 2 tau up to ~53)
-constexpr int kAngSlots = kAngNMax / 32;
 constexpr int kAngBuildSlots = 6;      // table nodes: up to 192 partial waves
 
-template <class T> struct AngConst;
-template <> struct AngConst<double> {
+// Scaling limits of the recurrences.
+struct AngConst {
   static constexpr double big = 1e280, grow = 1e100, shrink = 1e-100, shrink2 = 1e-200, seed = 1e-30;
-};
-template <> struct AngConst<float> {
-  static constexpr float big = 1e30f, grow = 1e15f, shrink = 1e-15f, shrink2 = 1e-30f, seed = 1e-10f;
 };
 
 __device__ __forceinline__ double ang_sin(double x) { return sin(x); }
 __device__ __forceinline__ float ang_sin(float x) { return sinf(x); }
 __device__ __forceinline__ double ang_cos(double x) { return cos(x); }
 __device__ __forceinline__ float ang_cos(float x) { return cosf(x); }
-__device__ __forceinline__ double ang_y0(double x) { return y0(x); }
-__device__ __forceinline__ float ang_y0(float x) { return y0f(x); }
-__device__ __forceinline__ double ang_y1(double x) { return y1(x); }
-__device__ __forceinline__ float ang_y1(float x) { return y1f(x); }
 
 // First kind, orders 0..N, by the downward recurrence from M = N + 40 + z (spherical: sum rule
 // sum (2n+1) j_n^2 = 1, sign of j_0 or j_1; cylindrical: J_0 + 2 sum J_2k = 1).
-template <class T>
-__device__ __forceinline__ void bessel_first(int dim, int N, T z, T* __restrict__ j) {
-  using C = AngConst<T>;
+__device__ __forceinline__ void bessel_first(int dim, int N, double z, double* __restrict__ j) {
+  using C = AngConst;
   int M = N + 40 + (int)z;
   if (dim == 2 && (M & 1)) ++M;
-  T jp1 = T(0), jn = C::seed, sum = T(0);
-  T scale_acc = T(1);   // product of rescalings applied to the stored values
-  (void)scale_acc;
+  double jp1 = 0.0, jn = C::seed, sum = 0.0;
 #pragma unroll 1
   for (int n = M; n >= 0; --n) {
     if (n <= N) j[n] = jn;
-    sum += dim == 3 ? T(2 * n + 1) * jn * jn : (n == 0 ? jn : ((n & 1) ? T(0) : T(2) * jn));
-    const T jm1 = n > 0 ? (dim == 3 ? T(2 * n + 1) : T(2 * n)) / z * jn - jp1 : T(0);
+    sum += dim == 3 ? (double)(2 * n + 1) * jn * jn : (n == 0 ? jn : ((n & 1) ? 0.0 : 2.0 * jn));
+    const double jm1 = n > 0 ? (dim == 3 ? (double)(2 * n + 1) : (double)(2 * n)) / z * jn - jp1 : 0.0;
     jp1 = jn;
     jn = jm1;
     if (fabs(jn) > C::grow) {
@@ -77,40 +66,29 @@ __device__ __forceinline__ void bessel_first(int dim, int N, T z, T* __restrict_
       sum *= dim == 3 ? C::shrink2 : C::shrink;
     }
   }
-  T scale;
+  double scale;
   if (dim == 3) {
-    scale = T(1) / sqrt(sum);
-    const T s = ang_sin(z), c = ang_cos(z);
-    const T j0 = s / z, j1 = s / (z * z) - c / z;
-    const bool neg = fabs(j0) >= fabs(j1) ? ((j0 < T(0)) != (j[0] < T(0))) : ((j1 < T(0)) != (j[1] < T(0)));
+    scale = 1.0 / sqrt(sum);
+    const double s = sin(z), c = cos(z);
+    const double j0 = s / z, j1 = s / (z * z) - c / z;
+    const bool neg = fabs(j0) >= fabs(j1) ? ((j0 < 0.0) != (j[0] < 0.0)) : ((j1 < 0.0) != (j[1] < 0.0));
     if (neg) scale = -scale;
   } else {
-    scale = T(1) / sum;
+    scale = 1.0 / sum;
   }
   for (int n = 0; n <= N; ++n) j[n] *= scale;
 }
 
 // Second kind of orders 0 and 1 at z.
-template <class T>
-__device__ __forceinline__ void bessel_second01(int dim, T z, T& y0v, T& y1v) {
+__device__ __forceinline__ void bessel_second01(int dim, double z, double& y0v, double& y1v) {
   if (dim == 3) {
-    const T s = ang_sin(z), c = ang_cos(z);
+    const double s = sin(z), c = cos(z);
     y0v = -c / z;
     y1v = -c / (z * z) - s / z;
   } else {
-    y0v = ang_y0(z);
-    y1v = ang_y1(z);
+    y0v = y0(z);
+    y1v = y1(z);
   }
-}
-
-// lane-distributed value of slot k (k < S) of the partial-wave coefficients
-template <class T, int S>
-__device__ __forceinline__ T ang_slot(const T (&acc)[S], int k) {
-  T v = acc[0];
-#pragma unroll
-  for (int s = 1; s < S; ++s)
-    if (k == s) v = acc[s];
-  return v;
 }
 
 // partial waves the law of concentration kappa needs (the series' terms beyond are below 1e-16)
@@ -126,88 +104,64 @@ __device__ __forceinline__ T warp_sum(T v) {
   return v;
 }
 
-// CDF of the conditional angle at v from the distributed coefficients (every lane returns it).
-template <class T, int S>
-__device__ __forceinline__ T ang_cdf_warp(int dim, const T (&acc)[S], T inv_d0, int N, T v) {
-  const int lane = threadIdx.x & 31;
-  T part = T(0);
-  if (dim == 3) {
-    // sum_{n>=1} (D_n/D_0) [P_{n+1}(v) - P_{n-1}(v)] / 2 : every lane runs the recurrence and adds its orders
-    T pm1 = T(1), p = v;   // P_{n-1}, P_n at n = 1
-#pragma unroll 1
-    for (int n = 1; n <= N; ++n) {
-      const T pp1 = (T(2 * n + 1) * v * p - T(n) * pm1) / T(n + 1);
-      if ((n & 31) == lane) part += ang_slot(acc, n >> 5) * (pp1 - pm1);
-      pm1 = p;
-      p = pp1;
-    }
-    return T(0.5) * (T(1) + v) + T(0.5) * inv_d0 * warp_sum(part);
-  }
-  // 2D: [theta + 2 sum_{n>=1} (D_n/D_0) sin(n theta)/n] / pi
-#pragma unroll 1
-  for (int n = lane; n <= N; n += 32)
-    if (n >= 1) part += ang_slot(acc, n >> 5) * ang_sin(T(n) * v) / T(n);
-  return (v + T(2) * inv_d0 * warp_sum(part)) / T(kPi);
-}
-
 // Partial-wave integrals D_0 .. D_N (N < 32 S) of the law at (R, R0, tau), lane-distributed: lane l
 // holds D_{l + 32 s} in acc[s].  Warp-collective.
-template <class T, int S>
-__device__ __forceinline__ void ang_coeffs_warp(int dim, int N, T R, T R0, T tau, const double* __restrict__ gl16,
-                                                T (&acc)[S]) {
-  using C = AngConst<T>;
+template <int S>
+__device__ __forceinline__ void ang_coeffs_warp(int dim, int N, double R, double R0, double tau, const double* __restrict__ gl16,
+                                                double (&acc)[S]) {
+  using C = AngConst;
   const int lane = threadIdx.x & 31;
-  const T X = sqrt(T(46) / tau);
-  const int panels = 8 + (int)ceil(X * (R + R0) / T(1.5));
+  const double X = sqrt(46.0 / tau);
+  const int panels = 8 + (int)ceil(X * (R + R0) / 1.5);
   const int nodes = 16 * panels;
   // 3D: panels in x on [0, X]; 2D: in t with x = t^2 on [0, sqrt(X)] (dx = 2t dt), which smooths the
   // logarithmic behaviour of the integer-order boundary coefficients at x -> 0
-  const T hp = (dim == 3 ? X : sqrt(X)) / T(panels);
+  const double hp = (dim == 3 ? X : sqrt(X)) / panels;
 #pragma unroll
-  for (int s = 0; s < S; ++s) acc[s] = T(0);
-  T jx[32 * S + 2], jr[32 * S + 1], jq[32 * S + 1];
+  for (int s = 0; s < S; ++s) acc[s] = 0.0;
+  double jx[32 * S + 2], jr[32 * S + 1], jq[32 * S + 1];
 #pragma unroll 1
   for (int base = 0; base < nodes; base += 32) {
     const int k = base + lane;
     const bool on = k < nodes;
-    T w = T(0), x = T(1);
+    double w = 0.0, x = 1.0;
     // second kind: (y_n, y_{n+1}) at x, R x, R0 x, and y_{n-1} at x
-    T ax = T(0), bx = T(0), ar = T(0), br = T(0), aq = T(0), bq = T(0), px = T(0);
+    double ax = 0.0, bx = 0.0, ar = 0.0, br = 0.0, aq = 0.0, bq = 0.0, px = 0.0;
     if (on) {
       const int p = k >> 4, i = k & 15;
-      const T t = (T(p) + T(0.5)) * hp + T(0.5) * hp * T(gl16[i]);
+      const double t = (p + 0.5) * hp + 0.5 * hp * gl16[i];
       x = dim == 3 ? t : t * t;
-      w = T(0.5) * hp * T(gl16[16 + i]) * exp(-tau * x * x) * (dim == 3 ? x * x : x * T(2) * t);
-      bessel_first<T>(dim, N + 1, x, jx);
-      bessel_first<T>(dim, N, R * x, jr);
-      bessel_first<T>(dim, N, R0 * x, jq);
-      bessel_second01<T>(dim, x, ax, bx);
-      bessel_second01<T>(dim, R * x, ar, br);
-      bessel_second01<T>(dim, R0 * x, aq, bq);
+      w = 0.5 * hp * gl16[16 + i] * exp(-tau * x * x) * (dim == 3 ? x * x : x * 2.0 * t);
+      bessel_first(dim, N + 1, x, jx);
+      bessel_first(dim, N, R * x, jr);
+      bessel_first(dim, N, R0 * x, jq);
+      bessel_second01(dim, x, ax, bx);
+      bessel_second01(dim, R * x, ar, br);
+      bessel_second01(dim, R0 * x, aq, bq);
     }
     bool dead = !on;
 #pragma unroll 1
     for (int n = 0; n <= N; ++n) {
-      T c = T(0);
+      double c = 0.0;
       // an order whose second-kind values have grown past C::big contributes nothing here
       if (!dead && (fabs(bx) > C::big || fabs(ar) > C::big || fabs(aq) > C::big)) dead = true;
       if (!dead) {
-        const T kd = dim == 3 ? T(n + 1) : T(n);
-        const T jd = n == 0 ? -jx[1] : jx[n - 1] - kd / x * jx[n];
-        const T yd = n == 0 ? -bx : px - kd / x * ax;
-        T a = -x * jd, b = -x * yd;
-        T nr = fabs(b) > fabs(a) ? fabs(b) * sqrt(T(1) + (a / b) * (a / b)) : fabs(a) * sqrt(T(1) + (b / a) * (b / a));
-        const T car = a / nr, cbr = b / nr;
+        const double kd = dim == 3 ? (double)(n + 1) : (double)(n);
+        const double jd = n == 0 ? -jx[1] : jx[n - 1] - kd / x * jx[n];
+        const double yd = n == 0 ? -bx : px - kd / x * ax;
+        double a = -x * jd, b = -x * yd;
+        double nr = fabs(b) > fabs(a) ? fabs(b) * sqrt(1.0 + (a / b) * (a / b)) : fabs(a) * sqrt(1.0 + (b / a) * (b / a));
+        const double car = a / nr, cbr = b / nr;
         a = jx[n];
         b = ax;
-        nr = fabs(b) > fabs(a) ? fabs(b) * sqrt(T(1) + (a / b) * (a / b)) : fabs(a) * sqrt(T(1) + (b / a) * (b / a));
-        const T caa = a / nr, cba = b / nr;
-        const T ref = (jr[n] * cbr - ar * car) * (jq[n] * cbr - aq * car);
-        const T abs_ = (jr[n] * cba - ar * caa) * (jq[n] * cba - aq * caa);
+        nr = fabs(b) > fabs(a) ? fabs(b) * sqrt(1.0 + (a / b) * (a / b)) : fabs(a) * sqrt(1.0 + (b / a) * (b / a));
+        const double caa = a / nr, cba = b / nr;
+        const double ref = (jr[n] * cbr - ar * car) * (jq[n] * cbr - aq * car);
+        const double abs_ = (jr[n] * cba - ar * caa) * (jq[n] * cba - aq * caa);
         c = w * (ref - abs_);
         // advance: Z_{n+2} = (k_{n+1} / z) Z_{n+1} - Z_n, k_m = 2m + 1 (3D) or 2m (2D)
-        const T km = dim == 3 ? T(2 * n + 3) : T(2 * n + 2);
-        const T nx = km / x * bx - ax, nrr = km / (R * x) * br - ar, nq = km / (R0 * x) * bq - aq;
+        const double km = dim == 3 ? (double)(2 * n + 3) : (double)(2 * n + 2);
+        const double nx = km / x * bx - ax, nrr = km / (R * x) * br - ar, nq = km / (R0 * x) * bq - aq;
         px = ax;
         ax = bx;
         bx = nx;
@@ -224,31 +178,6 @@ __device__ __forceinline__ void ang_coeffs_warp(int dim, int N, T R, T R0, T tau
       }
     }
   }
-}
-
-// Angle of the new separation to the start separation at CDF value U: 3D cos(angle) in [-1, 1],
-// 2D the angle in [0, pi].  Returns NaN if the law needs more than kAngNMax partial waves.
-template <class T>
-__device__ __noinline__ T ang_sample_warp(int dim, T U, T R, T R0, T tau, const double* __restrict__ gl16) {
-  const T kappa = R * R0 / (T(2) * tau);
-  const int N = ang_terms(kappa);
-  if (N > kAngNMax - 1) return T(NAN);
-  T acc[kAngSlots];
-  ang_coeffs_warp<T, kAngSlots>(dim, N, R, R0, tau, gl16, acc);
-  const T d0 = __shfl_sync(0xFFFFFFFFu, acc[0], 0);
-  const T inv_d0 = T(1) / d0;
-  // bisection of the CDF to the last representable step
-  T lo = dim == 3 ? T(-1) : T(0), hi = dim == 3 ? T(1) : T(kPi);
-#pragma unroll 1
-  for (int it = 0; it < 200; ++it) {
-    const T mid = T(0.5) * (lo + hi);
-    if (mid <= lo || mid >= hi) break;
-    if (ang_cdf_warp<T>(dim, acc, inv_d0, N, mid) < U)
-      lo = mid;
-    else
-      hi = mid;
-  }
-  return T(0.5) * (lo + hi);
 }
 
 // A unit vector e1 perpendicular to the unit vector u (3D): the coordinate axis along u's smallest
@@ -290,17 +219,6 @@ __device__ __forceinline__ void ang_place(int dim, const T* u, T v, T U_azi, T* 
     dir[1] = s * u[0] + c * u[1];
     dir[2] = T(0);
   }
-}
-
-// The direction from the exact law, warp-collective; returns false (dir untouched) when the law
-// needs more partial waves than kAngNMax.
-template <class T>
-__device__ __forceinline__ bool ang_direction_warp(int dim, const T* u, T U_ang, T U_azi, T Rn, T R0, T tau,
-                                                   const double* __restrict__ gl16, T* dir) {
-  const T v = ang_sample_warp<T>(dim, U_ang, Rn, R0, tau, gl16);
-  if (!(v == v)) return false;
-  ang_place<T>(dim, u, v, U_azi, dir);
-  return true;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -389,7 +307,7 @@ __device__ __forceinline__ void ang_table_node(int dim, double R, double R0, dou
   double kref = kappa;
   if (N <= 32 * kAngBuildSlots - 1) {
     double acc[kAngBuildSlots];
-    ang_coeffs_warp<double, kAngBuildSlots>(dim, N, R, R0, tau, gl16, acc);
+    ang_coeffs_warp<kAngBuildSlots>(dim, N, R, R0, tau, gl16, acc);
     const double inv_d0 = 1.0 / __shfl_sync(0xFFFFFFFFu, acc[0], 0);
 #pragma unroll
     for (int k = 0; k < kAngBuildSlots; ++k) Dn[32 * k + lane] = acc[k] * inv_d0;

@@ -647,7 +647,7 @@ static cudaError_t autotune(rd_handle* h) {
   h->L.block = best_block;
   // one thread per (particle, stencil row) in the sweep, for small systems
   const int rows = h->cfg.dim == 3 ? 5 : (h->reach == 2 ? 3 : 2);
-  if (h->cfg.sweep_split == 0 && (double)h->L.cap_particles * rows < 4.0e9) {
+  if (h->cfg.sweep_split == 0 && h->L.sweep_split == 1 && (double)h->L.cap_particles * rows < 4.0e9) {
     h->L.sweep_split = rows;
     const int g_split = fused_grid_size(h->L, device_sms());
     const int fused0 = h->L.fused;
@@ -795,9 +795,13 @@ int rd_init(const rd_config* cfg, void* stream, rd_handle** out) {
   L.pdl = true;
   L.reach = h->reach;
   const int rows = c.dim == 3 ? 5 : (h->reach == 2 ? 3 : 2);
-  L.sweep_split = c.sweep_split == 2 && (double)cap * rows < 4.0e9 ? rows : 1;
+  // automatic: one sweep thread per particle, but per stencil row for FP64 in 2D, whose warps each
+  // evaluate the p_enc of their candidates together (fewer particles a warp: more SMs share the work)
+  const bool split = c.sweep_split == 2 || (c.sweep_split == 0 && c.dim == 2 && c.precision == RD_FP64);
+  L.sweep_split = split && (double)cap * rows < 4.0e9 ? rows : 1;
   L.match_grid = match_grid_for_current_device();
   L.precision = c.precision;
+  L.dim = c.dim;
   L.block = c.block_size > 0 ? c.block_size : 256;
   L.max_grid = device_sms() * 16;
   // automatic: separate kernels under programmatic dependent launch, which measured faster than
@@ -1166,7 +1170,8 @@ int rd_resample(rd_handle* h, int32_t rule, const double* r0, const double* u, i
   if (!h || rule < 0 || rule >= h->cfg.n_pairs || n < 0 || (n > 0 && (!r0 || !u || !r_new))) return RD_EINVAL;
   if (h->cfg.pairs[rule].bc == RD_BC_NONE) return RD_EINVAL;
   if (n == 0) return RD_OK;
-  launch_resample(h->L.P, rule, r0, u, n, r_new, h->L.max_grid, h->stream);
+  launch_resample(h->L.P, rule, r0, u, n, r_new, h->cfg.precision == RD_FP64 && h->cfg.dim == 2, h->L.max_grid,
+                  h->stream);
   RD_CUDA(cudaGetLastError());
   return RD_OK;
 }
@@ -1176,7 +1181,7 @@ int rd_propagate(rd_handle* h, int32_t rule, const double* r0, const double* u, 
   const int bc = h->cfg.pairs[rule].bc;
   if (bc != RD_BC_REF && bc != RD_BC_RAD) return RD_EINVAL;
   if (n == 0) return RD_OK;
-  launch_propagate(h->L.P, rule, r0, u, n, r_out, h->L.max_grid, h->stream);
+  launch_propagate(h->L.P, rule, r0, u, n, r_out, h->hp.pairs[rule].tab_ang.v != nullptr, h->L.max_grid, h->stream);
   RD_CUDA(cudaGetLastError());
   return RD_OK;
 }
@@ -1514,6 +1519,7 @@ extern "C" int rd_step_static(const rd_config* cfg, void* stream, int64_t n, con
   L.sweep_split = 1;
   L.match_grid = match_grid_for_current_device();
   L.precision = c.precision;
+  L.dim = c.dim;
   L.block = 256;
   L.max_grid = device_sms() * 16;
   L.scan_items = 8;

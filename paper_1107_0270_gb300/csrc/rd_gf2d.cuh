@@ -247,45 +247,4 @@ __device__ __forceinline__ double cdf2(const Pair2D& q, double V, double R0, con
   return s * 0.5 * hstep;
 }
 
-// density 2 pi R (g_ref - g_abs) at R (derivative of cdf2)
-__device__ __forceinline__ double dens2(const Pair2D& q, double R, double R0) {
-  if (q.series) {
-    double ie[kSeriesTerms];
-    const double z = (R + R0 - 2.0) / (2.0 * q.s);
-    ierfc_scaled_all(z, kSeriesTerms, ie);
-    const double pref = exp(-z * z) / (4.0 * kPi * sqrt(q.tau * R * R0));
-    return 2.0 * kPi * R * pref * (series_bracket2(*q.ser, 1, R, R0, q.s, ie) + series_bracket2(*q.ser, 0, R, R0, q.s, ie));
-  }
-  double g[3];
-  weber_g(q.nodes, q.n_nodes, R, R0, 3u, g);
-  return 2.0 * kPi * R * (g[1] - g[0]);
-}
-
-// New separation R' >= 1 with tail fraction U (Newton on cdf2/tot = 1 - U within a bisection
-// bracket on (0, vmax), vmax = R0 + 13 sqrt(tau) beyond which the density is below e^{-40}).
-__device__ __forceinline__ double resample2(const Pair2D& q, double U, double R0, const double* __restrict__ gl16) {
-  if (R0 < 1.0) R0 = 1.0;
-  const double vmax = R0 + 13.0 * q.s;
-  const double tot = cdf2(q, vmax, R0, gl16);
-  const double target = (1.0 - U) * tot;
-  double lo = 0.0, hi = vmax, V = fmin(q.s, 0.5 * vmax);
-#pragma unroll 1
-  for (int it = 0; it < 100; ++it) {
-    const double f = cdf2(q, V, R0, gl16) - target;
-    if (f < 0.0)
-      lo = V;
-    else
-      hi = V;
-    const double d = dens2(q, 1.0 + V, R0);
-    double Vn = d > 0.0 ? V - f / d : 0.5 * (lo + hi);
-    const bool inside = Vn > lo && Vn < hi;
-    if (!inside) Vn = 0.5 * (lo + hi);
-    const double step = fabs(Vn - V);
-    V = Vn;
-    if (inside && step <= 1e-10 * fmax(V, q.s)) break;
-    if (hi - lo <= 4e-16 * fmax(hi, q.s)) break;
-  }
-  return 1.0 + V;
-}
-
 }  // namespace rd

@@ -416,6 +416,30 @@ __device__ __forceinline__ void lnT3_f(float V, float w, float s, float inv_4tau
   df = -(1.0f + V) * (q + 1.7724538509f * z * ey) / (s * 1.7724538509f * body);
 }
 
+// FP32 Newton solution V of ln T(V) = ln U (good to about 1e-5 of max(V, s)).
+__device__ __forceinline__ float resample3_seed(double U, double R0, double s) {
+  const float wf = (float)(R0 - 1.0), sf = (float)s, i4f = (float)(1.0 / (4.0 * s * s)), lnUf = (float)log(U);
+  const float lnx0f = logf(erfcxf(wf / (2.0f * sf)));
+  float Vf = 0.0f, lo = 0.0f, hi = -1.0f;
+  for (int it = 0; it < 24; ++it) {
+    float f, df;
+    lnT3_f(Vf, wf, sf, i4f, lnx0f, f, df);
+    const float g = f - lnUf;
+    if (g == 0.0f) break;
+    if (g > 0.0f)
+      lo = Vf;
+    else
+      hi = Vf;
+    float Vn = Vf - g / df;
+    const bool inside = Vn >= lo && (hi < 0.0f || Vn <= hi);
+    if (!inside) Vn = hi < 0.0f ? lo + fmaxf(lo, sf) : 0.5f * (lo + hi);
+    const float step = fabsf(Vn - Vf);
+    Vf = Vn;
+    if (inside && step <= 1e-5f * fmaxf(Vf, sf)) break;
+  }
+  return Vf >= 0.0f && isfinite(Vf) ? Vf : 0.0f;
+}
+
 // Solves ln T(V) = ln U.  A few FP32 Newton steps give a seed good to ~1e-5; FP64 Newton steps,
 // each kept inside the bracket known so far (bisection / expansion otherwise), finish the solve.
 // Once an FP64 Newton step is below 1e-10 of the length scale max(V, s), quadratic convergence
@@ -425,30 +449,7 @@ __device__ __forceinline__ double resample3(double U, double R0, double s) {
   const double w = R0 - 1.0;
   const double inv_4tau = 1.0 / (4.0 * s * s);
   const double lnU = log(U);
-  // FP32 seed
-  float Vf = 0.0f;
-  {
-    const float wf = (float)w, sf = (float)s, i4f = (float)inv_4tau, lnUf = (float)lnU;
-    const float lnx0f = logf(erfcxf(wf / (2.0f * sf)));
-    float lo = 0.0f, hi = -1.0f;
-    for (int it = 0; it < 24; ++it) {
-      float f, df;
-      lnT3_f(Vf, wf, sf, i4f, lnx0f, f, df);
-      const float g = f - lnUf;
-      if (g == 0.0f) break;
-      if (g > 0.0f)
-        lo = Vf;
-      else
-        hi = Vf;
-      float Vn = Vf - g / df;
-      const bool inside = Vn >= lo && (hi < 0.0f || Vn <= hi);
-      if (!inside) Vn = hi < 0.0f ? lo + fmaxf(lo, sf) : 0.5f * (lo + hi);
-      const float step = fabsf(Vn - Vf);
-      Vf = Vn;
-      if (inside && step <= 1e-5f * fmaxf(Vf, sf)) break;
-    }
-    if (!(Vf >= 0.0f) || !isfinite(Vf)) Vf = 0.0f;
-  }
+  const float Vf = resample3_seed(U, R0, s);
   const double ln_ex0 = log(erfcx(w / (2.0 * s)));
   double lo = 0.0, hi = -1.0;          // hi < 0: no upper bound yet
   double V = (double)Vf, f = 0.0, df;

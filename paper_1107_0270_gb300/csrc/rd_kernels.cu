@@ -9,6 +9,7 @@
 
 #include "rd_angle.cuh"
 #include "rd_gf2d.cuh"
+#include "rd_laplace.cuh"
 #include "rd_kernels.h"
 
 namespace rd {
@@ -83,17 +84,22 @@ __device__ __forceinline__ Pair2D pair2d(const PairDev& pr) {
 }
 __device__ __noinline__ double p_enc2_call(const PairDev& pr, double R, double R0) { return p_enc2(pair2d(pr), R, R0); }
 __device__ __noinline__ double p_reac2_call(const PairDev& pr, double R, double R0) { return p_reac2(pair2d(pr), R, R0); }
-__device__ __noinline__ double resample2_call(const DevParams& P, const PairDev& pr, double U, double R0) {
-  return resample2(pair2d(pr), U, R0, P.gl16);
-}
 __device__ __forceinline__ double p_enc_dim(const DevParams& P, const PairDev& pr, double R, double R0) {
   return P.dim == 3 ? p_enc3(R, R0, pr.inv_tau) : p_enc2_call(pr, R, R0);
 }
 __device__ __forceinline__ double p_reac_dim(const DevParams& P, const PairDev& pr, double R, double R0) {
   return P.dim == 3 ? p_reac3(R, R0, pr.s, pr.alpha) : p_reac2_call(pr, R, R0);
 }
+// 2D: warp-collective, every lane with the same arguments (the law's nodes are shared by the lanes);
+// 3D: per thread.
 __device__ __forceinline__ double resample_dim(const DevParams& P, const PairDev& pr, double U, double R0) {
-  return P.dim == 3 ? resample3(U, R0, pr.s) : resample2_call(P, pr, U, R0);
+  if (P.dim == 3) return resample3(U, R0, pr.s);
+  return lap_resample2_warp(U, R0, pr.tau, (double)resample3_seed(U, fmax(R0, 1.0), pr.s));
+}
+
+// p_reac of the step's resolution: 2D warp-collective like resample_dim, 3D per thread.
+__device__ __forceinline__ double p_reac_item(const DevParams& P, const PairDev& pr, double R, double R0) {
+  return P.dim == 3 ? p_reac3(R, R0, pr.s, pr.alpha) : lap_p_reac2_warp(R, R0, pr.tau, pr.h);
 }
 
 // ================================================================================================
@@ -495,6 +501,77 @@ __device__ __forceinline__ void ph_sweep(const DevParams* Pp, DevCtl* ctl,
   uint2* queue = s_queue[threadIdx.x >> 5];
   uint32_t qc = 0;   // entries in this warp's queue (the same in every lane)
   unsigned long long n_cand = 0, n_near = 0, n_overlap = 0;
+  uint2* eval_q = nullptr;    // FP64 step in 2D: pairs left to the warp (at most the 32 of one pass)
+  uint32_t* eval_n = nullptr;
+  if constexpr (sizeof(T) == 8) {
+    __shared__ uint2 s_eval[8][32];
+    __shared__ uint32_t s_neval[8];
+    eval_q = s_eval[threadIdx.x >> 5];
+    eval_n = &s_neval[threadIdx.x >> 5];
+    if (lane == 0) *eval_n = 0u;
+    __syncwarp();
+  }
+
+  // A fired pair (k, jj) to the list; swap: jj holds the lower id.
+  auto append = [&](const uint32_t k, const uint32_t jj, const bool swap, const uint32_t id_lo, const uint32_t id_hi,
+                    const int rule, const uint32_t r, const double p, const double key) {
+    const unsigned m = __activemask();
+    const int leader = __ffs(m) - 1;
+    uint32_t base = 0;
+    if (lane == leader) base = atomicAdd(&ctl->fired, (uint32_t)__popc(m));
+    base = __shfl_sync(m, base, leader);
+    const uint32_t pos = base + __popc(m & ((1u << lane) - 1u));
+    if (pos < cap_pairs) {
+      FiredPair f;
+      const uint32_t ia = sidx[k], ib = sidx[jj];
+      f.ia = swap ? ib : ia;
+      f.ib = swap ? ia : ib;
+      f.ida = id_lo;
+      f.idb = id_hi;
+      f.p = p;
+      f.key = key;
+      fired[pos] = f;
+      fstate[pos] = FS_LIVE | ((uint32_t)rule << 2) | (r << 8);
+      matched[f.ia] = -1;
+      matched[f.ib] = -1;
+      atomicAdd(&deg[f.ia], 1u);
+      atomicAdd(&deg[f.ib], 1u);
+    } else {
+      set_status(ctl, RD_ECAPACITY);
+    }
+  };
+
+  // FP64 step in 2D: the queued pairs whose p_enc the whole warp evaluates, one after the other.
+  auto drain = [&]() {
+    if constexpr (sizeof(T) == 8) {
+      __syncwarp();
+      const uint32_t ne = *(volatile uint32_t*)eval_n;
+      for (uint32_t q = 0; q < ne; ++q) {
+        const uint2 e = eval_q[q];
+        const auto a0 = sx0[2 * (size_t)e.x], a1 = sx1[2 * (size_t)e.x], b0 = sx0[2 * (size_t)e.y],
+                   b1 = sx1[2 * (size_t)e.y];
+        const uint32_t wa = w_bits(a0.w), r = wa >> 8, ida = w_bits(a1.w), idb = w_bits(b1.w);
+        const RepDev& rep = reps[r];
+        const int rule = P.pair_of[wa & 0xFFu][w_bits(b0.w) & 0xFFu];
+        const PairDev& pr = P.pairs[rule];
+        const double r0x = min_image(b0.x - a0.x, rep.L, rep.half_L), r0y = min_image(b0.y - a0.y, rep.L, rep.half_L);
+        const double rx = min_image(b1.x - a1.x, rep.L, rep.half_L), ry = min_image(b1.y - a1.y, rep.L, rep.half_L);
+        const double p = lap_p_enc2_warp(sqrt(norm2_rn(rx, ry, 0.0, 2)) / pr.sigma,
+                                         sqrt(norm2_rn(r0x, r0y, 0.0, 2)) / pr.sigma, pr.tau);
+        const bool swap = idb < ida;
+        const uint32_t id_lo = swap ? idb : ida, id_hi = swap ? ida : idb;
+        const uint4 w = draw(P, step, id_lo, id_hi, TAG_ENC, r);
+        const double u_enc = u52(w.x, w.y);
+        if (lane == 0) {
+          n_near += fabs(u_enc - p) <= 1e-9;
+          if (u_enc < p) append(e.x, e.y, swap, id_lo, id_hi, rule, r, p, -log(u52(w.z, w.w)) / p);
+        }
+        __syncwarp();
+      }
+      if (lane == 0) *eval_n = 0u;
+      __syncwarp();
+    }
+  };
 
   // One candidate pair (k, jj) within the cut-off: p_enc, the encounter draw, the append.
   auto process = [&](const uint32_t k, const uint32_t jj) {
@@ -544,6 +621,17 @@ __device__ __forceinline__ void ph_sweep(const DevParams* Pp, DevCtl* ctl,
           const double R0 = sqrt(r02) / pr.sigma;
           const double R = sqrt(norm2_rn(rx, ry, rz, dim)) / pr.sigma;
           overlap = R <= 1.0;
+          if (dim == 2 && !pr.series2d) {
+            // 2D beyond the small-time series: a pair fires only if its draw lies below p_enc, and
+            // p_enc below its closed bound; the few pairs whose draw is under the bound are
+            // evaluated by the whole warp (drain), the others are done
+            ++n_cand;
+            n_overlap += overlap;
+            const uint4 w = draw(P, step, id_lo, id_hi, TAG_ENC, r);
+            if (u52(w.x, w.y) < (double)p_enc2_bound(R, R0, pr.inv_tau))
+              eval_q[atomicAdd(eval_n, 1u)] = make_uint2(k, jj);
+            return;
+          }
           p = p_enc_dim(P, pr, R, R0);
         } else {
           const float rx = min_image_f(b1.x - a1.x, rep.Lf, rep.half_Lf);
@@ -579,34 +667,12 @@ __device__ __forceinline__ void ph_sweep(const DevParams* Pp, DevCtl* ctl,
           fires = u23(w.x) < pf;
         }
         if (fires) {
-          const unsigned m = __activemask();
-          const int lane = threadIdx.x & 31;
-          const int leader = __ffs(m) - 1;
-          uint32_t base = 0;
-          if (lane == leader) base = atomicAdd(&ctl->fired, (uint32_t)__popc(m));
-          base = __shfl_sync(m, base, leader);
-          const uint32_t pos = base + __popc(m & ((1u << lane) - 1u));
-          if (pos < cap_pairs) {
-            FiredPair f;
-            const uint32_t ia = sidx[k], ib = sidx[jj];
-            f.ia = swap ? ib : ia;
-            f.ib = swap ? ia : ib;
-            f.ida = id_lo;
-            f.idb = id_hi;
-            f.p = p;
-            if constexpr (sizeof(T) == 8)
-              f.key = -log(u52(w.z, w.w)) / p;
-            else
-              f.key = (double)(-logf(u23(w.z)) / pf);
-            fired[pos] = f;
-            fstate[pos] = FS_LIVE | ((uint32_t)rule << 2) | (r << 8);
-            matched[f.ia] = -1;
-            matched[f.ib] = -1;
-            atomicAdd(&deg[f.ia], 1u);
-            atomicAdd(&deg[f.ib], 1u);
-          } else {
-            set_status(ctl, RD_ECAPACITY);
-          }
+          double key;
+          if constexpr (sizeof(T) == 8)
+            key = -log(u52(w.z, w.w)) / p;
+          else
+            key = (double)(-logf(u23(w.z)) / pf);
+          append(k, jj, swap, id_lo, id_hi, rule, r, p, key);
         }
   };
 
@@ -731,6 +797,7 @@ __device__ __forceinline__ void ph_sweep(const DevParams* Pp, DevCtl* ctl,
         qc -= 32;
         __syncwarp();
         process(e.x, e.y);
+        drain();
       }
     }
   }
@@ -740,13 +807,14 @@ __device__ __forceinline__ void ph_sweep(const DevParams* Pp, DevCtl* ctl,
     const uint2 e = queue[lane];
     process(e.x, e.y);
   }
+  drain();
   warp_sum_add(&ctl->stats[RD_STAT_CANDIDATES], n_cand);
   warp_sum_add(&ctl->stats[RD_STAT_NEAR_THRESHOLD], n_near);
   warp_sum_add(&ctl->stats[RD_STAT_OVERLAPS], n_overlap);
 }
 
 template <class T, bool kSplit, int kReach>
-__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 4 : 5) k_sweep(const DevParams* __restrict__ Pp, DevCtl* __restrict__ ctl,
+__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 5) k_sweep(const DevParams* __restrict__ Pp, DevCtl* __restrict__ ctl,
                                                   const RepDev* __restrict__ reps,
                                                   const typename V4<T>::type* __restrict__ sx0,
                                                   const typename V4<T>::type* __restrict__ sx1,
@@ -935,7 +1003,7 @@ __device__ __forceinline__ void resolve_pair(const DevParams& P, const RepDev* r
                                              typename V4<T>::type* x1, uint32_t* status,
                                              typename V4<T>::type* prodpos, unsigned long long& n_react,
                                              unsigned long long& n_res, unsigned long long& n_near,
-                                             DevCtl* ctl, AngJob* jobs, uint32_t job_cap) {
+                                             DevCtl* ctl, AngJob* jobs, uint32_t job_cap, bool lead) {
   const int dim = P.dim;
     const uint32_t fs = fstate[e];
     const FiredPair f = fired[e];
@@ -1012,18 +1080,19 @@ __device__ __forceinline__ void resolve_pair(const DevParams& P, const RepDev* r
           b1[d] = wrap(c[d] + cb * nr, rep.L);
         }
       }
-      ++n_res;
+      n_res += lead;
       if (pr.bc == RD_BC_RAD) {
         const double pf = dim == 3 ? (double)p_reac3_f((float)Rn, (float)R0, pr.s_f, pr.alpha_f) : -1.0;
         if (dim == 3 && fabs(u_reac - pf) > kFilter) {
           react = u_reac < pf;
         } else {
-          const double p = p_reac_dim(P, pr, Rn, R0);
-          n_near += fabs(u_reac - p) <= 1e-9;
+          const double p = p_reac_item(P, pr, Rn, R0);
+          n_near += lead && fabs(u_reac - p) <= 1e-9;
           react = u_reac < p;
         }
       }
     }
+    if (!lead) return;      // a warp's other lanes shared the evaluations above
     if (react) {
       ++n_react;
       uint32_t np = 0;
@@ -1055,7 +1124,7 @@ __device__ __forceinline__ void decay_products(const DevParams& P, const RepDev*
                                                const uint32_t* id, uint32_t* status,
                                                typename V4<T>::type* prodpos, unsigned long long& n_rec,
                                                unsigned long long& n_near, DevCtl* ctl,
-                                               AngJob* jobs, uint32_t job_cap) {
+                                               AngJob* jobs, uint32_t job_cap, bool lead) {
   const int dim = P.dim;
     const uint32_t st = status[i];
     const DecayDev& dc = P.decays[(st >> ST_CHANNEL_SHIFT) & 15u];
@@ -1072,6 +1141,7 @@ __device__ __forceinline__ void decay_products(const DevParams& P, const RepDev*
       const double ell = sqrt(2.0 * P.D[dc.p0] * P.dt);
       double q3[3] = {0, 0, 0};
       for (int d = 0; d < dim; ++d) q3[d] = wrap(xp[d] + ell * nr[d], rep.L);
+      if (!lead) return;
       put4<T>(&prodpos[2 * (size_t)i], q3, pack_sp((uint32_t)dc.p0, r));
       np = 1;
     } else if (dc.n_products == 2) {
@@ -1114,8 +1184,8 @@ __device__ __forceinline__ void decay_products(const DevParams& P, const RepDev*
           if (dim == 3 && fabs(u_reac - pf) > kFilter) {
             recombine = u_reac < pf;
           } else {
-            const double p = p_reac_dim(P, pr, Rn, 1.0);
-            n_near += fabs(u_reac - p) <= 1e-9;
+            const double p = p_reac_item(P, pr, Rn, 1.0);
+            n_near += lead && fabs(u_reac - p) <= 1e-9;
             recombine = u_reac < p;
           }
         }
@@ -1144,7 +1214,7 @@ __device__ __forceinline__ void decay_products(const DevParams& P, const RepDev*
           aj.wa = pack_sp((uint32_t)sa, r);
           aj.wb = pack_sp((uint32_t)sb, r);
           aj.r = r;
-          push_ang_job(ctl, jobs, job_cap, aj);
+          if (lead) push_ang_job(ctl, jobs, job_cap, aj);
         }
       } else {
         double nr[4];
@@ -1152,6 +1222,7 @@ __device__ __forceinline__ void decay_products(const DevParams& P, const RepDev*
         const double ellr = sqrt(2.0 * Drel * P.dt);
         for (int d = 0; d < dim; ++d) rv[d] = dc.sigma_place * dir[d] + ellr * nr[d];
       }
+      if (!lead) return;    // a warp's other lanes shared the evaluations above
       if (recombine) {
         ++n_rec;
         if (product >= 0) {
@@ -1173,7 +1244,7 @@ __device__ __forceinline__ void decay_products(const DevParams& P, const RepDev*
         np = 2;
       }
     }
-    status[i] = st | (np << ST_NPROD_SHIFT);
+    if (lead) status[i] = st | (np << ST_NPROD_SHIFT);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1563,8 +1634,8 @@ __device__ __forceinline__ void replica_table(int n_replicas, const RepDev* reps
   if (threadIdx.x == 0) ctl->n_new = (uint32_t)(carry >> 32) + (uint32_t)carry;
 }
 
-// One accepted pair or one decay of this step (item q of the combined list).
-// One accepted pair or one decay of this step (item q of the combined list).
+// One accepted pair or one decay of this step (item q of the combined list), by one thread, or (FP64
+// step in 2D) by a warp whose lanes share the law's nodes, lead marking the lane that writes.
 template <class T>
 __device__ __noinline__ void resolve_item(const DevParams& P, const RepDev* reps,
                                              const FiredPair* fired, const uint32_t* fstate,
@@ -1575,13 +1646,14 @@ __device__ __noinline__ void resolve_item(const DevParams& P, const RepDev* reps
                                              uint32_t* rep_cons, uint32_t* rep_prod,
                                              unsigned long long& n_react, unsigned long long& n_res,
                                              unsigned long long& n_rec, unsigned long long& n_near,
-                                             DevCtl* ctl, AngJob* jobs, uint32_t job_cap) {
+                                             DevCtl* ctl, AngJob* jobs, uint32_t job_cap, bool lead) {
   if constexpr (sizeof(T) == 8) {
     if (pair)
       resolve_pair<T>(P, reps, fired, fstate, idx, step, x0, x1, status, prodpos, n_react, n_res, n_near, ctl, jobs,
-                      job_cap);
+                      job_cap, lead);
     else
-      decay_products<T>(P, reps, idx, step, x0, id, status, prodpos, n_rec, n_near, ctl, jobs, job_cap);
+      decay_products<T>(P, reps, idx, step, x0, id, status, prodpos, n_rec, n_near, ctl, jobs, job_cap, lead);
+    if (!lead) return;
   } else {
     if (pair)
       resolve_pair_f(P, reps, fired, fstate, idx, step, x0, x1, status, prodpos, n_react, n_res, ctl, jobs, job_cap);
@@ -1635,7 +1707,13 @@ __device__ __forceinline__ void ph_match_resolve(
   // n_accept holds the trivially accepted pairs only: the rounds count theirs in n_round_acc, so
   // every block reads the same n_triv whenever it starts
   const uint32_t nc = ctl->n_conflict, n_triv = ctl->n_accept, nd = ctl->n_decay, step = ctl->step;
-  const bool multi = nc > P.match_single_max && gridDim.x > 1;
+  // FP64 step in 2D: a warp resolves an item, consecutive items go to different blocks (the FP64
+  // pipe of an SM is what a resolution waits for), and with any conflicts at all the rounds run on the
+  // whole grid so that the pairs they accept are spread as well
+  const bool by_warp = sizeof(T) == 8 && P.dim == 2;
+  const bool lead = !by_warp || (threadIdx.x & 31) == 0;
+  const uint32_t wpb = blockDim.x >> 5, wid = threadIdx.x >> 5;
+  const bool multi = nc > (by_warp ? 0u : P.match_single_max) && gridDim.x > 1;
   unsigned long long n_react = 0, n_res = 0, n_near = 0, n_rec = 0;
   if (!multi) {
     // block 0 runs the (short) rounds alone, the other blocks resolve meanwhile
@@ -1643,10 +1721,11 @@ __device__ __forceinline__ void ph_match_resolve(
     const uint32_t nblk = skip0 ? gridDim.x - 1 : gridDim.x;
     if (!(skip0 && blockIdx.x == 0)) {
       const uint32_t b = skip0 ? blockIdx.x - 1 : blockIdx.x;
-      for (uint32_t q = b * blockDim.x + threadIdx.x; q < n_triv + nd; q += nblk * blockDim.x) {
+      const uint32_t q0 = by_warp ? wid * nblk + b : b * blockDim.x + threadIdx.x;
+      for (uint32_t q = q0; q < n_triv + nd; q += nblk * (by_warp ? wpb : blockDim.x)) {
         const bool pair = q < n_triv;
         resolve_item<T>(P, reps, fired, fstate, pair, pair ? accepted[q] : decay_list[q - n_triv], step, x0, x1, id,
-                        status, prodpos, rep_cons, rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap);
+                        status, prodpos, rep_cons, rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap, lead);
       }
     }
   }
@@ -1654,9 +1733,9 @@ __device__ __forceinline__ void ph_match_resolve(
     // short list: block 0 matches in shared memory, then resolves the pairs it accepted
     if (match_rounds_smem(P, ctl, fired, fstate, matched, conflict, accepted, nc, n_triv)) {
       const uint32_t n_acc = n_triv + *(volatile uint32_t*)&ctl->n_round_acc;
-      for (uint32_t q = n_triv + threadIdx.x; q < n_acc; q += blockDim.x)
+      for (uint32_t q = n_triv + (by_warp ? wid : threadIdx.x); q < n_acc; q += by_warp ? wpb : blockDim.x)
         resolve_item<T>(P, reps, fired, fstate, true, accepted[q], step, x0, x1, id, status, prodpos, rep_cons,
-                        rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap);
+                        rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap, lead);
     }
   } else if (nc > 0 && (multi || blockIdx.x == 0)) {
     const uint32_t nthr = multi ? gridDim.x * blockDim.x : blockDim.x;
@@ -1761,10 +1840,11 @@ __device__ __forceinline__ void ph_match_resolve(
     if (ok) {
       const uint32_t n_acc = n_triv + *(volatile uint32_t*)&ctl->n_round_acc;
       const uint32_t first = multi ? 0u : n_triv, last = multi ? n_acc + nd : n_acc;
-      for (uint32_t q = first + tid; q < last; q += nthr) {
+      const uint32_t q0 = !by_warp ? tid : (multi ? wid * gridDim.x + blockIdx.x : wid);
+      for (uint32_t q = first + q0; q < last; q += by_warp ? nthr >> 5 : nthr) {
         const bool pair = q < n_acc;
         resolve_item<T>(P, reps, fired, fstate, pair, pair ? accepted[q] : decay_list[q - n_acc], step, x0, x1, id,
-                        status, prodpos, rep_cons, rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap);
+                        status, prodpos, rep_cons, rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap, lead);
       }
     }
   }
@@ -1837,14 +1917,15 @@ __device__ __forceinline__ void ang_job_place(const AngJob& j, const RepDev& rep
 // Angle pass: the new separation direction of every encountered pair and every decay's product
 // pair that the resolution left to it (angle mode 0), then the particles placed.  Mixed step: one
 // thread per job from the rule's tabulated law; jobs of rules without a table (and every job of the
-// FP64 step) one warp per job from the full propagator (the partial-wave evaluation is
-// warp-collective).
+// FP64 step) one warp per job from the full propagator (rd_laplace.cuh), consecutive jobs in
+// different blocks: the FP64 pipe of an SM is the bound, about 28 000 cycles a job in 3D.
 template <class T>
 __device__ __forceinline__ void ph_angles(const DevParams* Pp, DevCtl* ctl,
                                           const RepDev* reps, const AngJob* jobs,
                                           uint32_t job_cap, typename V4<T>::type* x1,
                                           typename V4<T>::type* prodpos, const uint32_t bid,
                                           const uint32_t nblk) {
+  __shared__ double s_dn[8][kAngNMax];
   const DevParams& P = *Pp;
   if (ctl->status) return;
   const uint32_t nj = min(ctl->n_ang, job_cap);
@@ -1866,17 +1947,20 @@ __device__ __forceinline__ void ph_angles(const DevParams* Pp, DevCtl* ctl,
       ang_job_place<T>(j, reps[j.r], dim, dir, x1, prodpos);
     }
   }
-  const uint32_t wpb = blockDim.x >> 5, nw = nblk * wpb;
-  const bool lane0 = (threadIdx.x & 31) == 0;
-  for (uint32_t q = bid * wpb + (threadIdx.x >> 5); q < nj; q += nw) {
+  const uint32_t wpb = blockDim.x >> 5, wid = threadIdx.x >> 5;
+  for (uint32_t q = wid * nblk + bid; q < nj; q += nblk * wpb) {
     const AngJob& j = jobs[q];
     if (sizeof(T) == 4 && P.pairs[j.kind >> 8].tab_ang.v) continue;
+    const double v = lap_ang_sample_warp(dim, j.U_ang, j.Rn, j.R0, j.tau, s_dn[wid]);
+    if ((threadIdx.x & 31) != 0) continue;
     T u[3] = {(T)j.u[0], (T)j.u[1], (T)j.u[2]}, dir[3];
-    if (!ang_direction_warp<T>(dim, u, (T)j.U_ang, (T)j.U_azi, (T)j.Rn, (T)j.R0, (T)j.tau, P.gl16, dir)) {
+    if (v == v) {
+      ang_place<T>(dim, u, (T)v, (T)j.U_azi, dir);
+    } else {
       for (int d = 0; d < 3; ++d) dir[d] = (T)j.fb[d];
-      n_fb += lane0;
+      ++n_fb;
     }
-    if (lane0) ang_job_place<T>(j, reps[j.r], dim, dir, x1, prodpos);
+    ang_job_place<T>(j, reps[j.r], dim, dir, x1, prodpos);
   }
   if (n_fb) atomicAdd(&ctl->stats[RD_STAT_ANGLE_FALLBACK], n_fb);
 }
@@ -2277,61 +2361,81 @@ __global__ void k_pair_probs(const DevParams* __restrict__ Pp, int rule, const d
   }
 }
 
-// Standalone propagation of encountered pairs (rd_propagate): one warp per pair, the same device
-// functions as the step (length from the radial law, direction from the partial-wave law).
-__global__ void k_propagate(const DevParams* __restrict__ Pp, int rule, const double* __restrict__ r0,
-                            const double* __restrict__ u, int64_t n, double* __restrict__ out) {
+// Start separation vector of pair k scaled by the contact radius, and its direction (x axis if zero).
+struct PropStart {
+  double u[3], R0;
+};
+__device__ __forceinline__ PropStart propagate_start(const PairDev& pr, int dim, const double* __restrict__ r0, int64_t k) {
+  const double a0 = r0[3 * k] / pr.sigma, a1 = r0[3 * k + 1] / pr.sigma, a2 = dim == 3 ? r0[3 * k + 2] / pr.sigma : 0.0;
+  const double l0 = sqrt(a0 * a0 + a1 * a1 + a2 * a2);
+  PropStart s = {{1.0, 0.0, 0.0}, l0 < 1.0 ? 1.0 : l0};
+  if (l0 > 0.0) {
+    s.u[0] = a0 / l0; s.u[1] = a1 / l0; s.u[2] = a2 / l0;
+  }
+  return s;
+}
+
+// Standalone propagation of encountered pairs (rd_propagate), the same device functions as the step.
+// Mixed handles: length and direction from the rule's tables, one thread per pair.
+__global__ void k_propagate_tab(const DevParams* __restrict__ Pp, int rule, const double* __restrict__ r0,
+                                const double* __restrict__ u, int64_t n, double* __restrict__ out) {
   const DevParams& P = *Pp;
   const PairDev& pr = P.pairs[rule];
   const int dim = P.dim;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n; k += nw) {
-    const double a0 = r0[3 * k] / pr.sigma, a1 = r0[3 * k + 1] / pr.sigma, a2 = dim == 3 ? r0[3 * k + 2] / pr.sigma : 0.0;
-    const double l0 = sqrt(a0 * a0 + a1 * a1 + a2 * a2);
-    const double R0 = l0 < 1.0 ? 1.0 : l0;
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
+    const PropStart s = propagate_start(pr, dim, r0, k);
+    const float Rn = resample_tab_ni(pr, dim == 3, (float)u[4 * k], (float)s.R0);
+    const float uu[3] = {(float)s.u[0], (float)s.u[1], (float)s.u[2]};
+    float dir[3] = {uu[0], uu[1], uu[2]};
+    const float v = ang_table_sample(pr.tab_ang, dim, (float)u[4 * k + 1], Rn, (float)s.R0);
+    if (v == v) ang_place<float>(dim, uu, v, (float)u[4 * k + 2], dir);
+    for (int d = 0; d < 3; ++d) out[3 * k + d] = d < dim ? (double)(Rn * dir[d]) * pr.sigma : 0.0;
+  }
+}
+
+// FP64 handles (and rules without an angle table): one warp per pair, direction from the full
+// propagator.
+__global__ void __launch_bounds__(32) k_propagate(const DevParams* __restrict__ Pp, int rule,
+                                                  const double* __restrict__ r0, const double* __restrict__ u,
+                                                  int64_t n, double* __restrict__ out) {
+  __shared__ double s_dn[kAngNMax];
+  const DevParams& P = *Pp;
+  const PairDev& pr = P.pairs[rule];
+  const int dim = P.dim;
+  for (int64_t k = blockIdx.x; k < n; k += gridDim.x) {
+    const PropStart s = propagate_start(pr, dim, r0, k);
     double res[3] = {0.0, 0.0, 0.0};
     if (P.precision == RD_MIXED) {
-      const float Rn = resample_tab_ni(pr, dim == 3, (float)u[4 * k], (float)R0);
-      float uu[3] = {1.0f, 0.0f, 0.0f}, dir[3];
-      if (l0 > 0.0) {
-        uu[0] = (float)(a0 / l0); uu[1] = (float)(a1 / l0); uu[2] = (float)(a2 / l0);
-      }
-      bool ok;
-      if (pr.tab_ang.v) {
-        // the mixed step's tabulated law
-        const float v = ang_table_sample(pr.tab_ang, dim, (float)u[4 * k + 1], Rn, (float)R0);
-        ok = v == v;
-        if (ok) ang_place<float>(dim, uu, v, (float)u[4 * k + 2], dir);
-      } else {
-        ok = ang_direction_warp<float>(dim, uu, (float)u[4 * k + 1], (float)u[4 * k + 2], Rn, (float)R0,
-                                       (float)pr.tau, P.gl16, dir);
-      }
-      if (!ok) {
-        dir[0] = uu[0]; dir[1] = uu[1]; dir[2] = uu[2];
-      }
+      const float Rn = resample_tab_ni(pr, dim == 3, (float)u[4 * k], (float)s.R0);
+      const double v = lap_ang_sample_warp(dim, u[4 * k + 1], Rn, s.R0, pr.tau, s_dn);
+      const float uu[3] = {(float)s.u[0], (float)s.u[1], (float)s.u[2]};
+      float dir[3] = {uu[0], uu[1], uu[2]};
+      if (v == v) ang_place<float>(dim, uu, (float)v, (float)u[4 * k + 2], dir);
       for (int d = 0; d < dim; ++d) res[d] = (double)(Rn * dir[d]);
     } else {
-      const double Rn = resample_dim_ni(P, pr, u[4 * k], R0);
-      double uu[3] = {1.0, 0.0, 0.0}, dir[3];
-      if (l0 > 0.0) {
-        uu[0] = a0 / l0; uu[1] = a1 / l0; uu[2] = a2 / l0;
-      }
-      if (!ang_direction_warp<double>(dim, uu, u[4 * k + 1], u[4 * k + 2], Rn, R0, pr.tau, P.gl16, dir)) {
-        dir[0] = uu[0]; dir[1] = uu[1]; dir[2] = uu[2];
-      }
+      const double Rn = resample_dim_ni(P, pr, u[4 * k], s.R0);
+      const double v = lap_ang_sample_warp(dim, u[4 * k + 1], Rn, s.R0, pr.tau, s_dn);
+      double dir[3] = {s.u[0], s.u[1], s.u[2]};
+      if (v == v) ang_place<double>(dim, s.u, v, u[4 * k + 2], dir);
       for (int d = 0; d < dim; ++d) res[d] = Rn * dir[d];
     }
-    if ((threadIdx.x & 31) == 0)
+    if (threadIdx.x == 0)
       for (int d = 0; d < 3; ++d) out[3 * k + d] = res[d] * pr.sigma;
   }
 }
 
+// One thread per draw, or (kWarp, FP64 handles in 2D) one warp.
+template <bool kWarp>
 __global__ void k_resample(const DevParams* __restrict__ Pp, int rule, const double* __restrict__ r0,
                            const double* __restrict__ u, int64_t n, double* __restrict__ out) {
   const PairDev& pr = Pp->pairs[rule];
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-    out[k] = (Pp->precision == RD_MIXED ? (double)resample_tab_ni(pr, Pp->dim == 3, (float)u[k], (float)(r0[k] / pr.sigma))
-                                        : resample_dim(*Pp, pr, u[k], r0[k] / pr.sigma)) * pr.sigma;
+  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t k = kWarp ? tid >> 5 : tid; k < n; k += kWarp ? nt >> 5 : nt) {
+    const double v = (!kWarp && Pp->precision == RD_MIXED
+                          ? (double)resample_tab_ni(pr, Pp->dim == 3, (float)u[k], (float)(r0[k] / pr.sigma))
+                          : resample_dim(*Pp, pr, u[k], r0[k] / pr.sigma)) * pr.sigma;
+    if (!kWarp || (threadIdx.x & 31) == 0) out[k] = v;
+  }
 }
 
 
@@ -2653,9 +2757,12 @@ static void step_impl(const StepLaunch& L, cudaStream_t s, KernelTimer* timer) {
            sx1, L.sidx);
   mark("k_scatter_cells");
   const uint32_t split = L.sweep_split > 1 ? (uint32_t)L.sweep_split : 1u;
-  const int Gs = grid_for(L.cap_particles * (int64_t)split, 256, L.max_grid);
+  // FP64 in 2D: one-warp blocks, so that the warp-wide p_enc evaluations (the FP64 pipe of an SM is
+  // what they wait for) spread over the SMs
+  const int Bs = sizeof(T) == 8 && L.dim == 2 ? 32 : 256;
+  const int Gs = grid_for(L.cap_particles * (int64_t)split, Bs, L.max_grid);
   auto sweep = [&](auto kernel) {
-    launch_k(pdl, kernel, Gs, 256, 0, s, L.P, L.ctl, L.reps, sx0, sx1, L.sidx, L.cell_start, L.total_cells, L.fired,
+    launch_k(pdl, kernel, Gs, Bs, 0, s, L.P, L.ctl, L.reps, sx0, sx1, L.sidx, L.cell_start, L.total_cells, L.fired,
              L.fstate, L.deg, L.matched, (uint32_t)L.cap_pairs, split);
   };
   if (L.reach == 2)
@@ -2876,13 +2983,19 @@ void launch_pair_probs(const DevParams* P, int rule, const double* r0, const dou
 }
 
 void launch_propagate(const DevParams* P, int rule, const double* r0, const double* u, int64_t n, double* out,
-                      int max_grid, cudaStream_t s) {
-  k_propagate<<<grid_for(n * 32, 128, max_grid), 128, 0, s>>>(P, rule, r0, u, n, out);
+                      bool table, int max_grid, cudaStream_t s) {
+  if (table)
+    k_propagate_tab<<<grid_for(n, 128, max_grid), 128, 0, s>>>(P, rule, r0, u, n, out);
+  else
+    k_propagate<<<grid_for(n, 1, max_grid), 32, 0, s>>>(P, rule, r0, u, n, out);
 }
 
 void launch_resample(const DevParams* P, int rule, const double* r0, const double* u, int64_t n, double* out,
-                     int max_grid, cudaStream_t s) {
-  k_resample<<<grid_for(n, 128, max_grid), 128, 0, s>>>(P, rule, r0, u, n, out);
+                     bool warp, int max_grid, cudaStream_t s) {
+  if (warp)
+    k_resample<true><<<grid_for(n, 1, max_grid), 32, 0, s>>>(P, rule, r0, u, n, out);
+  else
+    k_resample<false><<<grid_for(n, 128, max_grid), 128, 0, s>>>(P, rule, r0, u, n, out);
 }
 
 // Angle table of one pair rule (mixed step): one warp per node (a, b) of the law at

@@ -14,6 +14,7 @@ namespace rd {
 // Device buffers and sizes of one step (pointers are device addresses).
 struct StepLaunch {
   int precision;
+  int dim;
   int block;
   int max_grid;
   int scan_items;
@@ -123,13 +124,15 @@ void launch_pair_probs(const DevParams* P, int rule, const double* r0, const dou
 // kind 3 with fwd != nullptr: the 2D inverse table from the forward -ln(tail) table fwd
 void launch_build_table(const DevParams* P, int rule, int kind, float* out, float4* quad, int n0, int n1, double h,
                         double h1, double* tot, const Tab2* fwd, int device_sms, cudaStream_t s);
+// warp: one warp per draw (FP64 in 2D), else one thread
 void launch_resample(const DevParams* P, int rule, const double* r0, const double* u, int64_t n, double* out,
-                     int max_grid, cudaStream_t s);
+                     bool warp, int max_grid, cudaStream_t s);
 // Angle table of one pair rule into out (n0 x n1 x (kAngTabU + 3) floats), on stream s.
 void launch_build_ang_table(const DevParams* P, int dim, double tau, double h, int n0, int n1, float* out,
                             int device_sms, cudaStream_t s);
+// table: directions from the rule's angle table (mixed handles), else from the full propagator
 void launch_propagate(const DevParams* P, int rule, const double* r0, const double* u, int64_t n, double* out,
-                      int max_grid, cudaStream_t s);
+                      bool table, int max_grid, cudaStream_t s);
 
 // First-passage refinement of encountered pairs (one pair rule, one step length).
 constexpr int kFptMaxLevels = 24;
