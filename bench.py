@@ -171,10 +171,10 @@ def algorithmic_bytes(kernel, precision, w):
         "k_prepare": n * (2 * v + 16) + 4 * nb,
         # read the cell counts, write the cell starts, clear the counts
         "k_scan_cells": 12 * cells,
-        # read cell, slot, both positions, id, cell start; write both sorted positions + index
-        "k_scatter_cells": nb * (4 * v + 20),
-        # both positions of every binned particle once, the cell starts once, the fired records
-        "k_sweep": nb * 2 * v + 4 * cells + fired * 52,
+        # read cell, slot, start position, cell start; write the 16-byte sorted record
+        "k_scatter_cells": nb * (v + 28),
+        # the sorted record of every binned particle once, the cell starts once, the fired records
+        "k_sweep": nb * 16 + 4 * cells + fired * 52,
         # trivial pairs: fired records and both degrees, accepted / conflict lists (48 B per fired
         # pair); then degrees cleared, and per accepted pair or decay: record, state, 2x2 positions
         # read, 2 positions + statuses written (conflict rounds add re-reads of the conflict pairs)

@@ -256,6 +256,8 @@ static void derive_params(rd_handle* h) {
     P.pair_of[p.s1][p.s2] = (int8_t)k;
     P.pair_of[p.s2][p.s1] = (int8_t)k;
     P.binned_mask |= (1u << p.s1) | (1u << p.s2);
+    P.partners[p.s1] |= 1u << p.s2;
+    P.partners[p.s2] |= 1u << p.s1;
   }
   for (int sp = 0; sp < c.n_species; ++sp)
     for (int d = 0; d < 3; ++d) {
@@ -552,6 +554,16 @@ static int64_t layout_cells(const rd_config& c, const std::vector<rd_replica>& r
   return total;
 }
 
+// Squared radius of the sweep's FP32 cut-off test in a box of edge L.  The mixed step's FP32 positions
+// are the positions, so the test is the cut-off; the FP64 step tests rounded copies: each coordinate is
+// within 2^-24 L, a minimum-image difference within 2.4e-7 L, a length within 4.2e-7 L, its square
+// within 4e-7 relative of the FP64 one, all inside the margin (the FP64 test follows).
+static float screen_radius2(const DevParams& P, double rc, double L) {
+  if (P.precision == RD_MIXED) return P.rcut2_max_f;
+  const double r = rc * (1.0 + 1e-6) + 6e-7 * L;
+  return (float)(r * r);
+}
+
 // Cell-edge choice: a fixed factor (> 0) or the per-replica density rule with a multiplier (< 0).
 static cudaError_t apply_factor(rd_handle* h, double factor) {
   const rd_config& c = h->cfg;
@@ -676,6 +688,8 @@ static cudaError_t autotune(rd_handle* h) {
   }
   h->tuned_ms = best / 6.0;
   restore();
+  launch_count(launch_for(h, 0), h->stream);   // the trial steps moved the counts
+  cudaStreamSynchronize(h->stream);
   cudaEventDestroy(a);
   cudaEventDestroy(b);
   cudaFree(sx);
@@ -761,6 +775,7 @@ int rd_init(const rd_config* cfg, void* stream, rd_handle** out) {
     d.half_L = 0.5 * rp.L;
     d.Lf = (float)rp.L;
     d.half_Lf = 0.5f * d.Lf;
+    d.screen2 = screen_radius2(h->hp, rc, rp.L);
     int64_t nr = 0;
     for (int s = 0; s < c.n_species; ++s) nr += rp.n_init[s];
     d.beg = (uint32_t)n_total;
@@ -789,6 +804,7 @@ int rd_init(const rd_config* cfg, void* stream, rd_handle** out) {
   int64_t pair_cap = c.pair_capacity > 0 ? c.pair_capacity : std::max<int64_t>(65536, cap);
   h->hp.cap_particles = cap;
   h->hp.cap_pairs = pair_cap;
+  h->hp.rec_packed = cap <= (int64_t)kRecIndex;
 
   StepLaunch& L = h->L;
   std::memset(&L, 0, sizeof L);
@@ -808,7 +824,6 @@ int rd_init(const rd_config* cfg, void* stream, rd_handle** out) {
   // the fused launch on every workload timed (a grid barrier costs more than a kernel boundary the
   // next launch already overlaps); the autotuner tries the fused launch as well
   L.fused = c.step_launch == 1;
-  L.scan_items = 8;
   L.cap_particles = cap;
   L.cap_pairs = pair_cap;
   L.total_cells = total_cells;
@@ -816,8 +831,7 @@ int rd_init(const rd_config* cfg, void* stream, rd_handle** out) {
   L.fused_grid = fused_grid_size(L, device_sms());
   if (L.fused_grid < 1) L.fused = 0;
   cudaGetLastError();   // a refused attribute or occupancy query leaves no error behind
-  const int64_t chunk = 256 * (int64_t)L.scan_items;
-  const int64_t nbc = (max_cells + chunk - 1) / chunk, nbp = (cap + chunk - 1) / chunk;
+  const int64_t nbc = (max_cells + kScanTile - 1) / kScanTile, nbp = (cap + kCompactTile - 1) / kCompactTile;
   L.flag_stride = std::max(nbc, nbp) + 1;
 
   bool ok = true;
@@ -832,16 +846,13 @@ int rd_init(const rd_config* cfg, void* stream, rd_handle** out) {
   h->idbuf[0] = (uint32_t*)A(cap * 4);
   h->idbuf[1] = (uint32_t*)A(cap * 4);
   L.x1 = A(cap * vs);
-  // sorted start and end positions interleaved: record k's pair fills one 32-byte sector (mixed)
-  L.sx0 = A(2 * cap * vs);
-  L.sx1 = L.sx0 ? (void*)((char*)L.sx0 + vs) : nullptr;
   L.prodpos = A(2 * cap * vs);
   L.status = (uint32_t*)A(cap * 4);
   L.matched = (int32_t*)A(cap * 4);
   L.deg = (uint32_t*)A(cap * 4);
   L.cell_of = (uint32_t*)A(cap * 4);
   L.slot = (uint32_t*)A(cap * 4);
-  L.sidx = (uint32_t*)A(cap * 4);
+  L.rec = (float4*)A(cap * sizeof(float4));
   L.decay_list = (uint32_t*)A(cap * 4);
   L.best_key = (unsigned long long*)A(cap * 8);
   L.best_pid = (unsigned long long*)A(cap * 8);
@@ -866,6 +877,7 @@ int rd_init(const rd_config* cfg, void* stream, rd_handle** out) {
   L.angles = c.angle_mode == 0;
   L.ang_cap = L.angles ? (uint32_t)cap : 1u;
   L.ang_jobs = (AngJob*)A((size_t)L.ang_cap * sizeof(AngJob));
+  L.events = (uint2*)A(kMaxEvents * sizeof(uint2));
   L.counts = (unsigned long long*)A((size_t)L.n_counts * 8);
   L.history_len = kHistoryLen;
   L.history = (long long*)A((size_t)kHistoryLen * c.n_species * 8);
@@ -896,6 +908,8 @@ int rd_init(const rd_config* cfg, void* stream, rd_handle** out) {
   cudaError_t e = cudaSuccess;
   e = cudaMemsetAsync(L.cell_count, 0, max_cells * 4, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(L.deg, 0, cap * 4, h->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(L.best_key, 0xFF, cap * 8, h->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(L.best_pid, 0xFF, cap * 8, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(L.flags, 0, 2 * L.flag_stride * 4, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(L.status, 0, cap * 4, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(L.rep_cons, 0, (size_t)c.n_replicas * 4, h->stream);
@@ -1147,8 +1161,15 @@ int rd_set_state(rd_handle* h, int64_t n, const double* x, const int32_t* specie
   int32_t err = 0;
   RD_CUDA(cudaMemcpyAsync(&err, h->st_err, 4, cudaMemcpyDeviceToHost, s));
   RD_CUDA(cudaStreamSynchronize(s));
-  if (err) return RD_EINVAL;
+  if (err & 1) return RD_EINVAL;
   h->cur = spare;
+  if (err) {
+    // the replaced state had an aborted step: the matching's arrays may not be at rest
+    const size_t cap = (size_t)h->L.cap_particles;
+    RD_CUDA(cudaMemsetAsync(h->L.deg, 0, cap * 4, s));
+    RD_CUDA(cudaMemsetAsync(h->L.best_key, 0xFF, cap * 8, s));
+    RD_CUDA(cudaMemsetAsync(h->L.best_pid, 0xFF, cap * 8, s));
+  }
   // the counts of the new state follow in stream order (the next call that reads them synchronises)
   launch_count(launch_for(h, h->cur), s);
   RD_CUDA(cudaGetLastError());
@@ -1483,6 +1504,7 @@ extern "C" int rd_step_static(const rd_config* cfg, void* stream, int64_t n, con
   rep.half_L = 0.5 * rp.L;
   rep.Lf = (float)rp.L;
   rep.half_Lf = 0.5f * rep.Lf;
+  rep.screen2 = screen_radius2(tmp.hp, rc, rp.L);
   double factor = (c.cell_factor_x100 > 0 ? c.cell_factor_x100 : 100) / 100.0;
   int64_t cells = 1;
   for (int attempt = 0; attempt < 64; ++attempt) {
@@ -1511,6 +1533,7 @@ extern "C" int rd_step_static(const rd_config* cfg, void* stream, int64_t n, con
   const int64_t pair_cap = RD_STATIC_MAX_PAIRS;
   tmp.hp.cap_particles = cap;
   tmp.hp.cap_pairs = pair_cap;
+  tmp.hp.rec_packed = 1;
   const size_t vs = c.precision == RD_MIXED ? 16 : 32;
 
   StepLaunch L;
@@ -1522,28 +1545,26 @@ extern "C" int rd_step_static(const rd_config* cfg, void* stream, int64_t n, con
   L.dim = c.dim;
   L.block = 256;
   L.max_grid = device_sms() * 16;
-  L.scan_items = 8;
   L.cap_particles = cap;
   L.cap_pairs = pair_cap;
   L.total_cells = cells;
   L.n_counts = c.n_species;
-  const int64_t chunk = 256 * (int64_t)L.scan_items;
-  const int64_t nbc = (cells + chunk - 1) / chunk, nbp = (cap + chunk - 1) / chunk;
+  const int64_t nbc = (cells + kScanTile - 1) / kScanTile, nbp = (cap + kCompactTile - 1) / kCompactTile;
   Bump b{(unsigned char*)base};
   void* xb0 = b.take(cap * vs);
   void* xb1 = b.take(cap * vs);
   uint32_t* id0 = (uint32_t*)b.take(cap * 4);
   uint32_t* id1 = (uint32_t*)b.take(cap * 4);
   L.x1 = b.take(cap * vs);
-  L.sx0 = b.take(2 * cap * vs);
-  L.sx1 = (void*)((char*)L.sx0 + vs);
+  L.rec = (float4*)b.take(cap * sizeof(float4));
+  // unused: the sizes this entry point accepts stay those of its documented limits
+  b.take(2 * cap * vs - cap * sizeof(float4) + cap * 4 - kMaxEvents * sizeof(uint2));
   L.prodpos = b.take(2 * cap * vs);
   L.status = (uint32_t*)b.take(cap * 4);
   L.matched = (int32_t*)b.take(cap * 4);
   L.deg = (uint32_t*)b.take(cap * 4);
   L.cell_of = (uint32_t*)b.take(cap * 4);
   L.slot = (uint32_t*)b.take(cap * 4);
-  L.sidx = (uint32_t*)b.take(cap * 4);
   L.decay_list = (uint32_t*)b.take(cap * 4);
   L.best_key = (unsigned long long*)b.take(cap * 8);
   L.best_pid = (unsigned long long*)b.take(cap * 8);
@@ -1567,6 +1588,7 @@ extern "C" int rd_step_static(const rd_config* cfg, void* stream, int64_t n, con
   L.angles = c.angle_mode == 0;
   L.ang_cap = RD_STATIC_MAX_PARTICLES;
   L.ang_jobs = (AngJob*)b.take((size_t)L.ang_cap * sizeof(AngJob));
+  L.events = (uint2*)b.take(kMaxEvents * sizeof(uint2));
   L.counts = (unsigned long long*)b.take((size_t)L.n_counts * 8);
   L.P = (const DevParams*)b.take(sizeof(DevParams));
   L.ctl = (DevCtl*)b.take(sizeof(DevCtl));
@@ -1630,6 +1652,8 @@ extern "C" int rd_step_static(const rd_config* cfg, void* stream, int64_t n, con
   RD_CUDA(cudaMemsetAsync(L.cell_count, 0, (size_t)cells * 4, s));
   RD_CUDA(cudaMemsetAsync(L.flags, 0, (size_t)(2 * L.flag_stride) * 4, s));
   RD_CUDA(cudaMemsetAsync(L.deg, 0, (size_t)cap * 4, s));
+  RD_CUDA(cudaMemsetAsync(L.best_key, 0xFF, (size_t)cap * 8, s));
+  RD_CUDA(cudaMemsetAsync(L.best_pid, 0xFF, (size_t)cap * 8, s));
   RD_CUDA(cudaMemsetAsync(L.counts, 0, (size_t)L.n_counts * 8, s));
   RD_CUDA(cudaMemsetAsync(L.rep_cons, 0, 4, s));
   RD_CUDA(cudaMemsetAsync(L.rep_prod, 0, 4, s));

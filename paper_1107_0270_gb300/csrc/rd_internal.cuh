@@ -15,8 +15,9 @@ constexpr int kMaxDecays = RD_MAX_DECAYS;
 constexpr int kAngTabU = 64;       // intervals of the angle table's U axis
 constexpr int kAngTabStride = kAngTabU + 4;   // floats per (R0, R') node of the angle table
 constexpr uint32_t kNoCell = 0xFFFFFFFFu;
+constexpr uint32_t kRecIndex = 0x0FFFFFFFu;      // particle index in a packed cell-order record (species above)
 constexpr uint32_t kOneParticle = 0xFFFFFFFFu;   // id_b of one-particle random streams
-constexpr int kSmemCounts = 6144;                // per-block histogram of (replica, species) counts
+constexpr uint32_t kMaxEvents = 4096;            // consumed particles of a step that the event list holds
 
 // Random-stream tags (counter word 3, low byte; replica index in the upper 24 bits).
 enum Tag : uint32_t {
@@ -97,7 +98,7 @@ struct DevParams {
   double dt;
   uint32_t seed_lo, seed_hi;
   uint32_t binned_mask;        // species that appear in an interacting pair rule
-  uint32_t pad1;
+  uint32_t rec_packed;         // cell-order records carry the species in their index's upper 4 bits (capacity < 2^28)
   int64_t cap_particles, cap_pairs;
   double D[kMaxSpecies];
   float D_f[kMaxSpecies];
@@ -108,6 +109,7 @@ struct DevParams {
   unsigned long long uni_thr[kMaxSpecies];   // decay iff (52-bit draw m) < uni_thr
   double gl16[32];             // 16-point Gauss-Legendre nodes then weights on [-1, 1]
   int8_t pair_of[kMaxSpecies][kMaxSpecies];   // index into pairs, -1 = no interaction
+  uint32_t partners[kMaxSpecies];             // species each species interacts with, as a bit mask
   PairDev pairs[kMaxPairs];
   DecayDev decays[kMaxDecays];
   double rcut2_max;            // largest squared cut-off over the pair rules
@@ -124,7 +126,8 @@ struct RepDev {
   float inv_edge_f[3];
   int32_t nc[3];
   int64_t cell_base;
-  uint32_t beg, end, next_id, pad;
+  uint32_t beg, end, next_id;
+  float screen2;               // squared radius of the sweep's FP32 test (mixed: the largest cut-off)
 };
 
 struct DevCtl {
@@ -139,10 +142,13 @@ struct DevCtl {
   uint32_t n_ang;          // angle jobs of this step
   uint32_t epoch;          // incremented every step; tags the scan flags
   uint32_t tile_ctr[2];    // tile tickets of the two scans
+  uint32_t n_ev;           // consumed particles of this step (the event list holds the first kMaxEvents)
   uint32_t done_blocks;    // blocks of the compaction that finished
   uint32_t last_fired;     // fired pairs of the last completed step
   uint32_t bar_count;      // grid barrier of the cooperative matching: arrivals, generation
   uint32_t bar_gen;
+  uint32_t bar2_count;     // barrier of the blocks that run the conflict rounds
+  uint32_t bar2_gen;
   uint32_t live[2];        // live conflict pairs after a matching round (by round parity)
   uint32_t done_res;       // blocks of the matching / resolution kernel that finished
   uint32_t n_new;          // particles after this step (set with the replica table)
@@ -152,6 +158,7 @@ struct DevCtl {
   unsigned long long ph_acc[8];  // fused step: accumulated ns per phase
   double t;
   unsigned long long stats[RD_NSTATS];
+  long long tot[kMaxSpecies];    // particles of each species over all replicas
 };
 
 // Per-replica placement of this step's compaction (built once the resolution is complete):

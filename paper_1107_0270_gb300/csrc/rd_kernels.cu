@@ -65,6 +65,21 @@ __device__ __forceinline__ int cell_coord_f(float x, float inv_edge, int n) {
   int c = (int)(x * inv_edge);
   return c < 0 ? 0 : (c >= n ? n - 1 : c);
 }
+// Cell coordinates of a start position (z = 0 in 2D).
+template <class T>
+__device__ __forceinline__ int3 cell_coords(const typename V4<T>::type& p, const RepDev& rep, int dim) {
+  int3 c;
+  if constexpr (sizeof(T) == 8) {
+    c.x = cell_coord(p.x, rep.inv_edge[0], rep.nc[0]);
+    c.y = cell_coord(p.y, rep.inv_edge[1], rep.nc[1]);
+    c.z = dim == 3 ? cell_coord(p.z, rep.inv_edge[2], rep.nc[2]) : 0;
+  } else {
+    c.x = cell_coord_f(p.x, rep.inv_edge_f[0], rep.nc[0]);
+    c.y = cell_coord_f(p.y, rep.inv_edge_f[1], rep.nc[1]);
+    c.z = dim == 3 ? cell_coord_f(p.z, rep.inv_edge_f[2], rep.nc[2]) : 0;
+  }
+  return c;
+}
 
 
 // ------------------------------------------------------------------------------------------------
@@ -111,29 +126,32 @@ template <class T>
 __device__ __forceinline__ void ph_prepare(const DevParams* Pp, DevCtl* ctl,
                           const RepDev* reps, const typename V4<T>::type* x0,
                           const uint32_t* id, typename V4<T>::type* x1,
-                          uint32_t* status, uint32_t* cell_of, uint32_t* slot,
-                          uint32_t* cell_count, uint32_t* decay_list,
-                          unsigned long long* counts, int n_counts,
-                          typename V4<T>::type* x0d, const uint32_t bid, const uint32_t nblk) {
+                          uint32_t* status, uint32_t* cell_of, uint32_t* slot, uint32_t* cell_count, uint32_t* decay_list,
+                          typename V4<T>::type* x0d, const uint32_t cap, const uint32_t bid, const uint32_t nblk) {
   const DevParams& P = *Pp;
-  if (bid == 0) {
+  // the first particle's loads go out beside those of the control block
+  const uint32_t i0 = bid * blockDim.x + threadIdx.x;
+  typename V4<T>::type p_first{};
+  uint32_t id_first = 0;
+  if (i0 < cap) {
+    p_first = x0[i0];
+    id_first = id[i0];
+  }
+  if (bid == 0 && threadIdx.x == 0) {
     // counters of the step's later kernels (the counters used by this kernel were reset at the
     // end of the previous step)
-    for (int k = threadIdx.x; k < n_counts; k += blockDim.x) counts[k] = 0ull;
-    if (threadIdx.x == 0) {
-      ctl->epoch += 1u;
-      ctl->tile_ctr[0] = 0u;
-      ctl->tile_ctr[1] = 0u;
-    }
+    ctl->epoch += 1u;
+    ctl->tile_ctr[0] = 0u;
+    ctl->tile_ctr[1] = 0u;
   }
   if (ctl->status) return;
   const uint32_t n = ctl->n, step = ctl->step;
   const int dim = P.dim;
-  for (uint32_t i = bid * blockDim.x + threadIdx.x; i < n; i += nblk * blockDim.x) {
-    auto p = x0[i];
+  for (uint32_t i = i0; i < n; i += nblk * blockDim.x) {
+    auto p = i == i0 ? p_first : x0[i];
     const uint32_t wb = w_bits(p.w);
     const uint32_t sp = wb & 0xFFu, r = wb >> 8;
-    const uint32_t pid = id[i];
+    const uint32_t pid = i == i0 ? id_first : id[i];
     const RepDev& rep = reps[r];
     if (x0d) {
       // deterministic forces as a split step: the drift displacement first; the rest of the step
@@ -200,17 +218,8 @@ __device__ __forceinline__ void ph_prepare(const DevParams* Pp, DevCtl* ctl,
     x1[i] = q;
     uint32_t cell = kNoCell;
     if (!st && ((P.binned_mask >> sp) & 1u)) {
-      int cx, cy, cz = 0;
-      if constexpr (sizeof(T) == 8) {
-        cx = cell_coord(p.x, rep.inv_edge[0], rep.nc[0]);
-        cy = cell_coord(p.y, rep.inv_edge[1], rep.nc[1]);
-        if (dim == 3) cz = cell_coord(p.z, rep.inv_edge[2], rep.nc[2]);
-      } else {
-        cx = cell_coord_f(p.x, rep.inv_edge_f[0], rep.nc[0]);
-        cy = cell_coord_f(p.y, rep.inv_edge_f[1], rep.nc[1]);
-        if (dim == 3) cz = cell_coord_f(p.z, rep.inv_edge_f[2], rep.nc[2]);
-      }
-      cell = (uint32_t)(rep.cell_base + ((int64_t)cz * rep.nc[1] + cy) * rep.nc[0] + cx);
+      const int3 c = cell_coords<T>(p, rep, dim);
+      cell = (uint32_t)(rep.cell_base + ((int64_t)c.z * rep.nc[1] + c.y) * rep.nc[0] + c.x);
       slot[i] = atomicAdd(&cell_count[cell], 1u);
     }
     cell_of[i] = cell;
@@ -222,12 +231,11 @@ __global__ void k_prepare(const DevParams* __restrict__ Pp, DevCtl* __restrict__
                           const RepDev* __restrict__ reps, const typename V4<T>::type* __restrict__ x0,
                           const uint32_t* __restrict__ id, typename V4<T>::type* __restrict__ x1,
                           uint32_t* __restrict__ status, uint32_t* __restrict__ cell_of, uint32_t* __restrict__ slot,
-                          uint32_t* __restrict__ cell_count, uint32_t* __restrict__ decay_list,
-                          unsigned long long* __restrict__ counts, int n_counts,
-                          typename V4<T>::type* __restrict__ x0d) {
+                          uint32_t* __restrict__ cell_count,
+                          uint32_t* __restrict__ decay_list,
+                          typename V4<T>::type* __restrict__ x0d, const uint32_t cap) {
   pdl_enter();
-  ph_prepare<T>(Pp, ctl, reps, x0, id, x1, status, cell_of, slot, cell_count, decay_list, counts, n_counts, x0d,
-                blockIdx.x, gridDim.x);
+  ph_prepare<T>(Pp, ctl, reps, x0, id, x1, status, cell_of, slot, cell_count, decay_list, x0d, cap, blockIdx.x, gridDim.x);
 }
 
 // ================================================================================================
@@ -428,49 +436,53 @@ __global__ void __launch_bounds__(256) k_scan1(Load load, int64_t n_const, const
 }
 
 // ================================================================================================
-// K2: scatter of the binned particles into cell order: start-of-step position (w = species bits),
-// end-of-free-step position (w = id bits) and the particle index.
+// K2: scatter of the binned particles into cell order.  The record is 16 bytes: the start position in
+// FP32 and the particle's index (with its species where the index leaves room).  The sweep's walk reads
+// nothing else; the exact positions and ids of the few pairs that pass it are read through the index.
+// (A 32-byte start / end record and a separate index took 571 us on the 1e7-particle network.)
 // ================================================================================================
 template <class T>
-__device__ __forceinline__ void ph_scatter(const DevCtl* ctl, const typename V4<T>::type* x0,
-                                const typename V4<T>::type* x1, const uint32_t* id,
-                                const uint32_t* cell_of, const uint32_t* slot,
-                                const uint32_t* cell_start,
-                                typename V4<T>::type* sx0, typename V4<T>::type* sx1,
-                                uint32_t* sidx, const uint32_t bid, const uint32_t nblk) {
+__device__ __forceinline__ void ph_scatter(const DevParams* Pp, const DevCtl* ctl, const typename V4<T>::type* x0,
+                                const uint32_t* cell_of, const uint32_t* slot, const uint32_t* cell_start,
+                                float4* rec, const uint32_t cap, const uint32_t bid, const uint32_t nblk) {
+  const bool packed = Pp->rec_packed != 0;
+  const uint32_t i0 = bid * blockDim.x + threadIdx.x;
+  // the first particle's loads go out beside those of the control block
+  typename V4<T>::type p{};
+  uint32_t c = kNoCell, sl = 0;
+  if (i0 < cap) {
+    c = cell_of[i0];
+    sl = slot[i0];
+    p = x0[i0];
+  }
   if (ctl->status) return;
   const uint32_t n = ctl->n;
-  for (uint32_t i = bid * blockDim.x + threadIdx.x; i < n; i += nblk * blockDim.x) {
-    const uint32_t c = cell_of[i];
+  for (uint32_t i = i0; i < n; i += nblk * blockDim.x) {
+    if (i != i0) {
+      c = cell_of[i];
+      sl = slot[i];
+      p = x0[i];
+    }
     if (c == kNoCell) continue;
-    const uint32_t k = cell_start[c] + slot[i];
-    sx0[2 * (size_t)k] = x0[i];
-    auto q = x1[i];
-    if constexpr (sizeof(T) == 8)
-      q.w = w_from_bits_d(id[i]);
-    else
-      q.w = w_from_bits_f(id[i]);
-    sx1[2 * (size_t)k] = q;
-    sidx[k] = i;
+    const uint32_t link = packed ? i | ((w_bits(p.w) & 0xFFu) << 28) : i;
+    rec[cell_start[c] + sl] = make_float4((float)p.x, (float)p.y, (float)p.z, __uint_as_float(link));
   }
 }
 
 template <class T>
-__global__ void k_scatter_cells(const DevCtl* __restrict__ ctl, const typename V4<T>::type* __restrict__ x0,
-                                const typename V4<T>::type* __restrict__ x1, const uint32_t* __restrict__ id,
-                                const uint32_t* __restrict__ cell_of, const uint32_t* __restrict__ slot,
-                                const uint32_t* __restrict__ cell_start,
-                                typename V4<T>::type* __restrict__ sx0, typename V4<T>::type* __restrict__ sx1,
-                                uint32_t* __restrict__ sidx) {
+__global__ void k_scatter_cells(const DevParams* __restrict__ Pp, const DevCtl* __restrict__ ctl,
+                                const typename V4<T>::type* __restrict__ x0, const uint32_t* __restrict__ cell_of,
+                                const uint32_t* __restrict__ slot, const uint32_t* __restrict__ cell_start,
+                                float4* __restrict__ rec, const uint32_t cap) {
   pdl_enter();
-  ph_scatter<T>(ctl, x0, x1, id, cell_of, slot, cell_start, sx0, sx1, sidx, blockIdx.x, gridDim.x);
+  ph_scatter<T>(Pp, ctl, x0, cell_of, slot, cell_start, rec, cap, blockIdx.x, gridDim.x);
 }
 
 // ================================================================================================
 // K3: cell sweep.  One thread per binned particle (cell order) walks the forward half of the
-// 27-cell (3D) / 9-cell (2D) neighbourhood; every pair (k, j > k) of an interacting species pair
-// whose start-of-step minimum-image distance is below r_cut is a candidate: p_enc from the start and
-// end separations, U_enc < p_enc fires and the pair is appended with a warp-aggregated atomic.
+// 27-cell (3D) / 9-cell (2D) neighbourhood; every pair of an interacting species pair whose
+// start-of-step minimum-image distance is below r_cut is a candidate: p_enc from the start and end
+// separations, U_enc < p_enc fires and the pair is appended with a warp-aggregated atomic.
 // In cell order the three cells x-1..x+1 of a row are one contiguous particle range, so the half
 // stencil is five row ranges (3D: own row from k+1 through x+1, row y+1, the three rows of layer
 // z+1; 2D: the first two), each split in two where the row wraps around x.
@@ -480,16 +492,15 @@ constexpr int kSweepRanges = 10;
 template <class T, bool kSplit, int kReach>
 __device__ __forceinline__ void ph_sweep(const DevParams* Pp, DevCtl* ctl,
                                          const RepDev* reps,
-                                         const typename V4<T>::type* sx0,
-                                         const typename V4<T>::type* sx1,
-                                         const uint32_t* sidx,
+                                         const typename V4<T>::type* x0,
+                                         const typename V4<T>::type* x1,
+                                         const uint32_t* id, const float4* rec,
                                          const uint32_t* cell_start,
                                          const int64_t total_cells, FiredPair* fired,
                                          uint32_t* fstate, uint32_t* deg,
                                          int32_t* matched, const uint32_t cap_pairs,
                                          const uint32_t split, uint2 (*ranges)[256],
                                          const uint32_t bid, const uint32_t nblk) {
-  using V = typename V4<T>::type;
   // per-warp queue of (particle, candidate) pairs that passed the cut-off test
   __shared__ uint2 s_queue[8][64];
   const DevParams& P = *Pp;
@@ -497,11 +508,12 @@ __device__ __forceinline__ void ph_sweep(const DevParams* Pp, DevCtl* ctl,
   const uint32_t nb = cell_start[total_cells];
   const uint32_t step = ctl->step;
   const int dim = P.dim;
+  const bool packed = P.rec_packed != 0;
   const int lane = threadIdx.x & 31;
   uint2* queue = s_queue[threadIdx.x >> 5];
   uint32_t qc = 0;   // entries in this warp's queue (the same in every lane)
   unsigned long long n_cand = 0, n_near = 0, n_overlap = 0;
-  uint2* eval_q = nullptr;    // FP64 step in 2D: pairs left to the warp (at most the 32 of one pass)
+  uint2* eval_q = nullptr;    // FP64 step: pairs that need the exact p_enc (at most the 32 of one pass)
   uint32_t* eval_n = nullptr;
   if constexpr (sizeof(T) == 8) {
     __shared__ uint2 s_eval[8][32];
@@ -523,9 +535,8 @@ __device__ __forceinline__ void ph_sweep(const DevParams* Pp, DevCtl* ctl,
     const uint32_t pos = base + __popc(m & ((1u << lane) - 1u));
     if (pos < cap_pairs) {
       FiredPair f;
-      const uint32_t ia = sidx[k], ib = sidx[jj];
-      f.ia = swap ? ib : ia;
-      f.ib = swap ? ia : ib;
+      f.ia = swap ? jj : k;
+      f.ib = swap ? k : jj;
       f.ida = id_lo;
       f.idb = id_hi;
       f.p = p;
@@ -541,145 +552,122 @@ __device__ __forceinline__ void ph_sweep(const DevParams* Pp, DevCtl* ctl,
     }
   };
 
-  // FP64 step in 2D: the queued pairs whose p_enc the whole warp evaluates, one after the other.
+  // FP64 step: the encounter decision of one queued pair from the exact p_enc (2D: by the whole warp, all
+  // lanes with the same pair; 3D: by this lane).
+  auto decide = [&](const uint2 e, const bool lead) {
+    if constexpr (sizeof(T) == 8) {
+      const auto a0 = x0[e.x], a1 = x1[e.x], b0 = x0[e.y], b1 = x1[e.y];
+      const uint32_t wa = w_bits(a0.w), r = wa >> 8, ida = id[e.x], idb = id[e.y];
+      const RepDev& rep = reps[r];
+      const int rule = P.pair_of[wa & 0xFFu][w_bits(b0.w) & 0xFFu];
+      const PairDev& pr = P.pairs[rule];
+      const double r0x = min_image(b0.x - a0.x, rep.L, rep.half_L), r0y = min_image(b0.y - a0.y, rep.L, rep.half_L);
+      const double rx = min_image(b1.x - a1.x, rep.L, rep.half_L), ry = min_image(b1.y - a1.y, rep.L, rep.half_L);
+      const double r0z = dim == 3 ? min_image(b0.z - a0.z, rep.L, rep.half_L) : 0.0;
+      const double rz = dim == 3 ? min_image(b1.z - a1.z, rep.L, rep.half_L) : 0.0;
+      const double R0 = sqrt(norm2_rn(r0x, r0y, r0z, dim)) / pr.sigma, R = sqrt(norm2_rn(rx, ry, rz, dim)) / pr.sigma;
+      const double p = dim == 3 ? p_enc3(R, R0, pr.inv_tau) : lap_p_enc2_warp(R, R0, pr.tau);
+      if (!lead) return;
+      // orient the pair from the lower id to the higher id
+      const bool swap = idb < ida;
+      const uint32_t id_lo = swap ? idb : ida, id_hi = swap ? ida : idb;
+      const uint4 w = draw(P, step, id_lo, id_hi, TAG_ENC, r);
+      const double u_enc = u52(w.x, w.y);
+      n_near += fabs(u_enc - p) <= 1e-9;
+      n_overlap += R <= 1.0;
+      if (u_enc < p) append(e.x, e.y, swap, id_lo, id_hi, rule, r, p, -log(u52(w.z, w.w)) / p);
+    }
+  };
   auto drain = [&]() {
     if constexpr (sizeof(T) == 8) {
       __syncwarp();
       const uint32_t ne = *(volatile uint32_t*)eval_n;
-      for (uint32_t q = 0; q < ne; ++q) {
-        const uint2 e = eval_q[q];
-        const auto a0 = sx0[2 * (size_t)e.x], a1 = sx1[2 * (size_t)e.x], b0 = sx0[2 * (size_t)e.y],
-                   b1 = sx1[2 * (size_t)e.y];
-        const uint32_t wa = w_bits(a0.w), r = wa >> 8, ida = w_bits(a1.w), idb = w_bits(b1.w);
-        const RepDev& rep = reps[r];
-        const int rule = P.pair_of[wa & 0xFFu][w_bits(b0.w) & 0xFFu];
-        const PairDev& pr = P.pairs[rule];
-        const double r0x = min_image(b0.x - a0.x, rep.L, rep.half_L), r0y = min_image(b0.y - a0.y, rep.L, rep.half_L);
-        const double rx = min_image(b1.x - a1.x, rep.L, rep.half_L), ry = min_image(b1.y - a1.y, rep.L, rep.half_L);
-        const double p = lap_p_enc2_warp(sqrt(norm2_rn(rx, ry, 0.0, 2)) / pr.sigma,
-                                         sqrt(norm2_rn(r0x, r0y, 0.0, 2)) / pr.sigma, pr.tau);
-        const bool swap = idb < ida;
-        const uint32_t id_lo = swap ? idb : ida, id_hi = swap ? ida : idb;
-        const uint4 w = draw(P, step, id_lo, id_hi, TAG_ENC, r);
-        const double u_enc = u52(w.x, w.y);
-        if (lane == 0) {
-          n_near += fabs(u_enc - p) <= 1e-9;
-          if (u_enc < p) append(e.x, e.y, swap, id_lo, id_hi, rule, r, p, -log(u52(w.z, w.w)) / p);
-        }
+      if (dim == 3) {
+        if (lane < (int)ne) decide(eval_q[lane], true);
         __syncwarp();
+      } else {
+        for (uint32_t q = 0; q < ne; ++q) {
+          decide(eval_q[q], lane == 0);
+          __syncwarp();
+        }
       }
       if (lane == 0) *eval_n = 0u;
       __syncwarp();
     }
   };
 
-  // One candidate pair (k, jj) within the cut-off: p_enc, the encounter draw, the append.
+  // One candidate pair (k, jj) within the sweep's test: its own cut-off, p_enc, the encounter draw, the
+  // append.
   auto process = [&](const uint32_t k, const uint32_t jj) {
-    const auto a0 = sx0[2 * (size_t)k];
-    const auto a1 = sx1[2 * (size_t)k];
+    const auto a0 = x0[k], a1 = x1[k];
     const uint32_t wa = w_bits(a0.w);
     const uint32_t spa = wa & 0xFFu, r = wa >> 8;
-    const uint32_t ida = w_bits(a1.w);
+    const uint32_t ida = id[k];
     const RepDev& rep = reps[r];
-    const auto b0 = sx0[2 * (size_t)jj];
-        // start-of-step separation first (the norm does not depend on the pair's orientation),
-        // against the largest cut-off; the species pair and its own cut-off after that
-        double p, r02;
-        float pf = 0.0f, r02f = 0.0f;
-        if constexpr (sizeof(T) == 8) {
-          const double r0x = min_image(b0.x - a0.x, rep.L, rep.half_L);
-          const double r0y = min_image(b0.y - a0.y, rep.L, rep.half_L);
-          const double r0z = dim == 3 ? min_image(b0.z - a0.z, rep.L, rep.half_L) : 0.0;
-          r02 = norm2_rn(r0x, r0y, r0z, dim);
-          if (!(r02 < P.rcut2_max)) return;
-        } else {
-          const float r0x = min_image_f(b0.x - a0.x, rep.Lf, rep.half_Lf);
-          const float r0y = min_image_f(b0.y - a0.y, rep.Lf, rep.half_Lf);
-          const float r0z = dim == 3 ? min_image_f(b0.z - a0.z, rep.Lf, rep.half_Lf) : 0.0f;
-          r02f = r0x * r0x + r0y * r0y + r0z * r0z;
-          if (!(r02f < P.rcut2_max_f)) return;
-        }
-        const uint32_t spb = w_bits(b0.w) & 0xFFu;
-        const int rule = P.pair_of[spa][spb];
-        if (rule < 0) return;
-        const PairDev& pr = P.pairs[rule];
-        if constexpr (sizeof(T) == 8) {
-          if (!(r02 < pr.rcut2)) return;
-        } else {
-          if (!(r02f < pr.rcut2_f)) return;
-        }
-        const auto b1 = sx1[2 * (size_t)jj];
-        const uint32_t idb = w_bits(b1.w);
-        // orient the pair from the lower id to the higher id
-        const bool swap = idb < ida;
-        const uint32_t id_lo = swap ? idb : ida, id_hi = swap ? ida : idb;
-        bool overlap;
-        if constexpr (sizeof(T) == 8) {
-          const double rx = min_image(b1.x - a1.x, rep.L, rep.half_L);
-          const double ry = min_image(b1.y - a1.y, rep.L, rep.half_L);
-          const double rz = dim == 3 ? min_image(b1.z - a1.z, rep.L, rep.half_L) : 0.0;
-          const double R0 = sqrt(r02) / pr.sigma;
-          const double R = sqrt(norm2_rn(rx, ry, rz, dim)) / pr.sigma;
-          overlap = R <= 1.0;
-          if (dim == 2 && !pr.series2d) {
-            // 2D beyond the small-time series: a pair fires only if its draw lies below p_enc, and
-            // p_enc below its closed bound; the few pairs whose draw is under the bound are
-            // evaluated by the whole warp (drain), the others are done
-            ++n_cand;
-            n_overlap += overlap;
-            const uint4 w = draw(P, step, id_lo, id_hi, TAG_ENC, r);
-            if (u52(w.x, w.y) < (double)p_enc2_bound(R, R0, pr.inv_tau))
-              eval_q[atomicAdd(eval_n, 1u)] = make_uint2(k, jj);
-            return;
-          }
-          p = p_enc_dim(P, pr, R, R0);
-        } else {
-          const float rx = min_image_f(b1.x - a1.x, rep.Lf, rep.half_Lf);
-          const float ry = min_image_f(b1.y - a1.y, rep.Lf, rep.half_Lf);
-          const float rz = dim == 3 ? min_image_f(b1.z - a1.z, rep.Lf, rep.half_Lf) : 0.0f;
-          const float d0 = (sqrtf(r02f) - pr.sigma_f) * pr.inv_sigma_f;
-          const float d = (sqrtf(rx * rx + ry * ry + rz * rz) - pr.sigma_f) * pr.inv_sigma_f;
-          overlap = d <= 0.0f;
-          if (dim == 3) {
-            pf = p_enc3_f(d, d0, pr.inv_tau_f);
-          } else if (d <= 0.0f || d0 <= 0.0f) {
-            pf = 1.0f;
-          } else {
-            const float xx = d * d0 * pr.inv_tau_f;
-            pf = xx > 60.0f ? 0.0f : fminf(1.0f, fmaxf(0.0f, tab_eval(pr.tab_penc, d0, d) * expf(-xx)));
-          }
-          p = (double)pf;
-        }
-        ++n_cand;
-        n_overlap += overlap;
-        // mixed step: FP32 draw and comparison; the smallest FP32 uniform is 2^-24, so a smaller
-        // p_enc cannot fire and needs no draw
-        if constexpr (sizeof(T) == 4) {
-          if (!(pf > 0x1p-24f)) return;
-        }
-        const uint4 w = draw(P, step, id_lo, id_hi, TAG_ENC, r);
-        bool fires;
-        if constexpr (sizeof(T) == 8) {
-          const double u_enc = u52(w.x, w.y);
-          n_near += fabs(u_enc - p) <= 1e-9;
-          fires = u_enc < p;
-        } else {
-          fires = u23(w.x) < pf;
-        }
-        if (fires) {
-          double key;
-          if constexpr (sizeof(T) == 8)
-            key = -log(u52(w.z, w.w)) / p;
-          else
-            key = (double)(-logf(u23(w.z)) / pf);
-          append(k, jj, swap, id_lo, id_hi, rule, r, p, key);
-        }
+    const auto b0 = x0[jj];
+    const int rule = P.pair_of[spa][w_bits(b0.w) & 0xFFu];
+    if (rule < 0) return;
+    const PairDev& pr = P.pairs[rule];
+    const auto b1 = x1[jj];
+    const uint32_t idb = id[jj];
+    // orient the pair from the lower id to the higher id
+    const bool swap = idb < ida;
+    const uint32_t id_lo = swap ? idb : ida, id_hi = swap ? ida : idb;
+    if constexpr (sizeof(T) == 8) {
+      // The cut-off is decided in FP64; then a pair fires only if its draw lies below p_enc, so the
+      // draw is compared with p_enc in FP32 (3D; in 2D with p_enc's closed bound) plus a margin over
+      // its rounding, and only the pairs below that, or as close to contact, take the FP64 evaluation.
+      const double r0x = min_image(b0.x - a0.x, rep.L, rep.half_L);
+      const double r0y = min_image(b0.y - a0.y, rep.L, rep.half_L);
+      const double r0z = dim == 3 ? min_image(b0.z - a0.z, rep.L, rep.half_L) : 0.0;
+      const double r02 = norm2_rn(r0x, r0y, r0z, dim);
+      if (!(r02 < pr.rcut2)) return;
+      const float rx = (float)min_image(b1.x - a1.x, rep.L, rep.half_L);
+      const float ry = (float)min_image(b1.y - a1.y, rep.L, rep.half_L);
+      const float rz = dim == 3 ? (float)min_image(b1.z - a1.z, rep.L, rep.half_L) : 0.0f;
+      ++n_cand;
+      const float d0 = (sqrtf((float)r02) - pr.sigma_f) * pr.inv_sigma_f;
+      const float d = (sqrtf(rx * rx + ry * ry + rz * rz) - pr.sigma_f) * pr.inv_sigma_f;
+      const uint4 w = draw(P, step, id_lo, id_hi, TAG_ENC, r);
+      const float u = __uint2float_rn(w.x) * 0x1p-32f;
+      if (d < 1e-3f || u < p_enc_screen(dim, d, d0, pr.inv_tau_f)) eval_q[atomicAdd(eval_n, 1u)] = make_uint2(k, jj);
+    } else {
+      const float r0x = min_image_f(b0.x - a0.x, rep.Lf, rep.half_Lf);
+      const float r0y = min_image_f(b0.y - a0.y, rep.Lf, rep.half_Lf);
+      const float r0z = dim == 3 ? min_image_f(b0.z - a0.z, rep.Lf, rep.half_Lf) : 0.0f;
+      const float r02f = r0x * r0x + r0y * r0y + r0z * r0z;
+      if (!(r02f < pr.rcut2_f)) return;
+      const float rx = min_image_f(b1.x - a1.x, rep.Lf, rep.half_Lf);
+      const float ry = min_image_f(b1.y - a1.y, rep.Lf, rep.half_Lf);
+      const float rz = dim == 3 ? min_image_f(b1.z - a1.z, rep.Lf, rep.half_Lf) : 0.0f;
+      const float d0 = (sqrtf(r02f) - pr.sigma_f) * pr.inv_sigma_f;
+      const float d = (sqrtf(rx * rx + ry * ry + rz * rz) - pr.sigma_f) * pr.inv_sigma_f;
+      float pf;
+      if (dim == 3) {
+        pf = p_enc3_f(d, d0, pr.inv_tau_f);
+      } else if (d <= 0.0f || d0 <= 0.0f) {
+        pf = 1.0f;
+      } else {
+        const float xx = d * d0 * pr.inv_tau_f;
+        pf = xx > 60.0f ? 0.0f : fminf(1.0f, fmaxf(0.0f, tab_eval(pr.tab_penc, d0, d) * expf(-xx)));
+      }
+      ++n_cand;
+      n_overlap += d <= 0.0f;
+      // FP32 draw and comparison; the smallest FP32 uniform is 2^-24, so a smaller p_enc cannot fire
+      // and needs no draw
+      if (!(pf > 0x1p-24f)) return;
+      const uint4 w = draw(P, step, id_lo, id_hi, TAG_ENC, r);
+      if (u23(w.x) < pf)
+        append(k, jj, swap, id_lo, id_hi, rule, r, (double)pf, (double)(-logf(u23(w.z)) / pf));
+    }
   };
 
   // Walks one particle's candidates and queues those within the cut-off; whenever the warp's
   // queue holds 32 pairs, all lanes process one each.  (Examining a candidate is cheap, processing
   // one is not: processed where it is found, the expensive part would run once per loop iteration
-  // in which any lane found one.)
+  // in which any lane found one.)  The walk reads the FP32 records only: in the mixed step they are the
+  // positions, in the FP64 step its test is a screen with a margin above the records' rounding, and
+  // process() decides.
   // split = 1: one thread walks all rows of a particle; split = number of rows: one thread per
   // (particle, row), more independent chains for small systems (the host keeps nb * split < 2^32)
   const uint32_t work = kSplit ? nb * split : nb;
@@ -688,11 +676,8 @@ __device__ __forceinline__ void ph_sweep(const DevParams* Pp, DevCtl* ctl,
   for (uint32_t it = 0; it < n_iter; ++it) {
     const uint32_t t = it * stride + bid * blockDim.x + threadIdx.x;
     int nr = 0;
-    uint32_t k = 0;
-    V a0{};
-    float4 cut{};   // (L, half L, largest squared cut-off) of the particle's replica, FP32 step
-    double Ld = 0.0, hLd = 0.0;
-    uint32_t spa = 0;
+    uint32_t k = 0, me = 0, mask = 0;
+    float ax = 0.0f, ay = 0.0f, az = 0.0f, Lf = 0.0f, hLf = 0.0f, cut = 0.0f;
     if (t < work) {
       k = kSplit ? t / split : t;
       const int row_lo = kSplit ? (int)(t - k * split) : 0;
@@ -700,21 +685,20 @@ __device__ __forceinline__ void ph_sweep(const DevParams* Pp, DevCtl* ctl,
       // cell edge >= r_cut / 2): rows y, y+1, y+2, each x-2 .. x+2 (own row x .. x+2)
       constexpr int kRows = kReach == 2 ? 3 : kSweepRanges / 2;
       const int row_hi = kSplit ? row_lo + 1 : kRows;
-      a0 = sx0[2 * (size_t)k];
-      const uint32_t wa = w_bits(a0.w);
-      spa = wa & 0xFFu;
-      const uint32_t r = wa >> 8;
-      const RepDev& rep = reps[r];
-      int cx, cy, cz = 0;
-      if constexpr (sizeof(T) == 8) {
-        cx = cell_coord(a0.x, rep.inv_edge[0], rep.nc[0]);
-        cy = cell_coord(a0.y, rep.inv_edge[1], rep.nc[1]);
-        if (dim == 3) cz = cell_coord(a0.z, rep.inv_edge[2], rep.nc[2]);
+      const float4 a = rec[k];
+      uint32_t wa = __float_as_uint(a.w);
+      me = packed ? wa & kRecIndex : wa;
+      int3 cc;
+      if (sizeof(T) == 4 && packed && P.n_replicas == 1) {
+        wa >>= 28;
+        if constexpr (sizeof(T) == 4) cc = cell_coords<float>(a, reps[0], dim);
       } else {
-        cx = cell_coord_f(a0.x, rep.inv_edge_f[0], rep.nc[0]);
-        cy = cell_coord_f(a0.y, rep.inv_edge_f[1], rep.nc[1]);
-        if (dim == 3) cz = cell_coord_f(a0.z, rep.inv_edge_f[2], rep.nc[2]);
+        const auto a0 = x0[me];
+        wa = w_bits(a0.w);
+        cc = cell_coords<T>(a0, reps[wa >> 8], dim);
       }
+      const RepDev& rep = reps[wa >> 8];
+      const int cx = cc.x, cy = cc.y, cz = cc.z;
       const int nc0 = rep.nc[0];
       // the grid has 1 or >= 2 kReach + 1 cells along each axis; with 1 only the own cell counts
       constexpr int kMinCells = 2 * kReach + 1;
@@ -742,9 +726,13 @@ __device__ __forceinline__ void ph_sweep(const DevParams* Pp, DevCtl* ctl,
           if (wrap_rg.y > wrap_rg.x) ranges[nr++][threadIdx.x] = wrap_rg;
         }
       }
-      Ld = rep.L;
-      hLd = rep.half_L;
-      cut = make_float4(rep.Lf, rep.half_Lf, 0.0f, 0.0f);
+      ax = a.x;
+      ay = a.y;
+      az = a.z;
+      Lf = rep.Lf;
+      hLf = rep.half_Lf;
+      cut = rep.screen2;
+      mask = P.partners[wa & 0xFFu];
     }
     int rr = 0;
     uint2 rg = nr > 0 ? ranges[0][threadIdx.x] : make_uint2(0u, 0u);
@@ -760,34 +748,16 @@ __device__ __forceinline__ void ph_sweep(const DevParams* Pp, DevCtl* ctl,
           rg = ranges[rr][threadIdx.x];
           j = rg.x;
         }
-        // the cut-off tests of process(), which repeats them
-        const auto b0 = sx0[2 * (size_t)jj];
-        bool in;
-        if constexpr (sizeof(T) == 8) {
-          const double r0x = min_image(b0.x - a0.x, Ld, hLd);
-          const double r0y = min_image(b0.y - a0.y, Ld, hLd);
-          const double r0z = dim == 3 ? min_image(b0.z - a0.z, Ld, hLd) : 0.0;
-          const double r02 = norm2_rn(r0x, r0y, r0z, dim);
-          in = r02 < P.rcut2_max;
-          if (in) {
-            const int rule = P.pair_of[spa][w_bits(b0.w) & 0xFFu];
-            in = rule >= 0 && r02 < P.pairs[rule].rcut2;
-          }
-        } else {
-          const float r0x = min_image_f(b0.x - a0.x, cut.x, cut.y);
-          const float r0y = min_image_f(b0.y - a0.y, cut.x, cut.y);
-          const float r0z = dim == 3 ? min_image_f(b0.z - a0.z, cut.x, cut.y) : 0.0f;
-          const float r02f = r0x * r0x + r0y * r0y + r0z * r0z;
-          in = r02f < P.rcut2_max_f;
-          if (in) {
-            const int rule = P.pair_of[spa][w_bits(b0.w) & 0xFFu];
-            in = rule >= 0 && r02f < P.pairs[rule].rcut2_f;
-          }
-        }
-        push = in;
+        const float4 b = rec[jj];
+        const uint32_t link = __float_as_uint(b.w);
+        jj = packed ? link & kRecIndex : link;
+        const uint32_t spb = packed ? link >> 28 : w_bits(x0[jj].w) & 0xFFu;
+        const float dx = min_image_f(b.x - ax, Lf, hLf), dy = min_image_f(b.y - ay, Lf, hLf);
+        const float dz = dim == 3 ? min_image_f(b.z - az, Lf, hLf) : 0.0f;
+        push = ((mask >> spb) & 1u) && dx * dx + dy * dy + dz * dz < cut;
       }
       const unsigned bal = __ballot_sync(0xFFFFFFFFu, push);
-      if (push) queue[qc + __popc(bal & ((1u << lane) - 1u))] = make_uint2(k, jj);
+      if (push) queue[qc + __popc(bal & ((1u << lane) - 1u))] = make_uint2(me, jj);
       qc += __popc(bal);
       __syncwarp();
       if (qc >= 32) {
@@ -814,11 +784,11 @@ __device__ __forceinline__ void ph_sweep(const DevParams* Pp, DevCtl* ctl,
 }
 
 template <class T, bool kSplit, int kReach>
-__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 5) k_sweep(const DevParams* __restrict__ Pp, DevCtl* __restrict__ ctl,
+__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 5) k_sweep(const DevParams* __restrict__ Pp, DevCtl* __restrict__ ctl,
                                                   const RepDev* __restrict__ reps,
-                                                  const typename V4<T>::type* __restrict__ sx0,
-                                                  const typename V4<T>::type* __restrict__ sx1,
-                                                  const uint32_t* __restrict__ sidx,
+                                                  const typename V4<T>::type* __restrict__ x0,
+                                                  const typename V4<T>::type* __restrict__ x1,
+                                                  const uint32_t* __restrict__ id, const float4* __restrict__ rec,
                                                   const uint32_t* __restrict__ cell_start,
                                                   const int64_t total_cells, FiredPair* __restrict__ fired,
                                                   uint32_t* __restrict__ fstate, uint32_t* __restrict__ deg,
@@ -826,7 +796,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 3 : 5) k_sweep(const Dev
                                                   const uint32_t split) {
   pdl_enter();
   __shared__ uint2 ranges[kSweepRanges][256];
-  ph_sweep<T, kSplit, kReach>(Pp, ctl, reps, sx0, sx1, sidx, cell_start, total_cells, fired, fstate, deg, matched,
+  ph_sweep<T, kSplit, kReach>(Pp, ctl, reps, x0, x1, id, rec, cell_start, total_cells, fired, fstate, deg, matched,
                               cap_pairs, split, ranges, blockIdx.x, gridDim.x);
 }
 
@@ -846,13 +816,19 @@ __device__ __forceinline__ void append_accepted(DevCtl* ctl, uint32_t* accepted,
   accepted[base + __popc(m & ((1u << lane) - 1u))] = e;
 }
 
+// FP32 keys (mixed step) fit one 64-bit word with the partner's id: at a shared particle the order (key,
+// partner id) is the order (key, id_a, id_b) of its pairs, so a minimum takes one atomic per endpoint.
+__device__ __forceinline__ unsigned long long key_bits_f(unsigned long long key) {
+  return (unsigned long long)__float_as_uint((float)__longlong_as_double((long long)key)) << 32;
+}
+
 __device__ __forceinline__ void ph_match_trivial(DevCtl* ctl, const FiredPair* fired,
                                 uint32_t* fstate, const uint32_t* deg,
                                 int32_t* matched, uint32_t* conflict,
                                 uint32_t* accepted,
                                 unsigned long long* best_key,
                                 unsigned long long* best_pid, uint32_t cap_pairs,
-                                ConflictRec* crec, const uint32_t bid, const uint32_t nblk) {
+                                ConflictRec* crec, const bool packed, const uint32_t bid, const uint32_t nblk) {
   if (ctl->status) return;
   const uint32_t nf = min(ctl->fired, cap_pairs);
   unsigned long long acc = 0;
@@ -885,10 +861,17 @@ __device__ __forceinline__ void ph_match_trivial(DevCtl* ctl, const FiredPair* f
         c.key = (unsigned long long)__double_as_longlong(f.key);
         c.pid = ((unsigned long long)f.ida << 32) | f.idb;
         crec[q] = c;
-        best_key[f.ia] = ~0ull;
-        best_key[f.ib] = ~0ull;
-        best_pid[f.ia] = ~0ull;
-        best_pid[f.ib] = ~0ull;
+        if (packed) {
+          // the first round's offers (both minima arrays are all ones between steps)
+          const unsigned long long kb = key_bits_f(c.key);
+          atomicMin(&best_key[f.ia], kb | f.idb);
+          atomicMin(&best_key[f.ib], kb | f.ida);
+        } else {
+          best_key[f.ia] = ~0ull;
+          best_key[f.ib] = ~0ull;
+          best_pid[f.ia] = ~0ull;
+          best_pid[f.ib] = ~0ull;
+        }
       }
     }
   }
@@ -907,21 +890,22 @@ constexpr uint32_t kBarrierSpin = 1u << 22;
 // arrival acquires every other block's arrival and releases the new generation, and each waiter
 // acquires the generation before the closing __syncthreads hands the data to its block.  Waiters
 // poll without sleeping for the first polls (the common wait is a few hundred nanoseconds).
-__device__ __forceinline__ bool grid_barrier(DevCtl* ctl, bool check_status = true) {
+__device__ __forceinline__ bool grid_barrier(DevCtl* ctl, bool check_status, uint32_t* count, uint32_t* gen,
+                                             uint32_t blocks) {
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
-    const uint32_t g = ld_acquire_gpu(&ctl->bar_gen);
+    const uint32_t g = ld_acquire_gpu(gen);
     int ok = 1;
     uint32_t old;
-    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(&ctl->bar_count) : "memory");
-    if (old == gridDim.x - 1) {
-      asm volatile("st.relaxed.gpu.global.u32 [%0], 0;" ::"l"(&ctl->bar_count) : "memory");
-      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&ctl->bar_gen) : "memory");
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(count) : "memory");
+    if (old == blocks - 1) {
+      asm volatile("st.relaxed.gpu.global.u32 [%0], 0;" ::"l"(count) : "memory");
+      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(gen) : "memory");
     } else {
       uint32_t spins = 0;
       const uint32_t limit = ctl->spin_limit ? ctl->spin_limit : kBarrierSpin;
-      while (ld_acquire_gpu(&ctl->bar_gen) == g) {
+      while (ld_acquire_gpu(gen) == g) {
         if (++spins > limit) {
           set_status(ctl, RD_ETIMEOUT);
           ok = 0;
@@ -939,6 +923,10 @@ __device__ __forceinline__ bool grid_barrier(DevCtl* ctl, bool check_status = tr
   }
   __syncthreads();
   return s_ok != 0;
+}
+// all blocks of the launch
+__device__ __forceinline__ bool grid_barrier(DevCtl* ctl, bool check_status = true) {
+  return grid_barrier(ctl, check_status, &ctl->bar_count, &ctl->bar_gen, gridDim.x);
 }
 
 // ================================================================================================
@@ -1646,7 +1634,8 @@ __device__ __noinline__ void resolve_item(const DevParams& P, const RepDev* reps
                                              uint32_t* rep_cons, uint32_t* rep_prod,
                                              unsigned long long& n_react, unsigned long long& n_res,
                                              unsigned long long& n_rec, unsigned long long& n_near,
-                                             DevCtl* ctl, AngJob* jobs, uint32_t job_cap, bool lead) {
+                                             DevCtl* ctl, AngJob* jobs, uint32_t job_cap, uint2* events,
+                                             bool lead) {
   if constexpr (sizeof(T) == 8) {
     if (pair)
       resolve_pair<T>(P, reps, fired, fstate, idx, step, x0, x1, status, prodpos, n_react, n_res, n_near, ctl, jobs,
@@ -1669,19 +1658,23 @@ __device__ __noinline__ void resolve_item(const DevParams& P, const RepDev* reps
     atomicAdd(&rep_cons[r], pair ? 2u : 1u);
     const uint32_t np = (st >> ST_NPROD_SHIFT) & 3u;
     if (np) atomicAdd(&rep_prod[r], np);
+    // the consumed particles (and the products of their owner) for the compaction
+    const uint32_t k = pair ? 2u : 1u, e = atomicAdd(&ctl->n_ev, k);
+    if (e + k <= kMaxEvents) {
+      events[e] = make_uint2(owner, np);
+      if (pair) events[e + 1] = make_uint2(fired[idx].ib, 0u);
+    }
   }
 }
 
 // K5: rounds of locally-dominant matching over the conflict list, and the resolution of every
 // accepted pair and every decay of the step (one cooperative launch).
-//  - A short conflict list is matched by block 0 alone (block barriers); trivially accepted pairs
-//    and decays involve no conflict pair, so blocks 1.. resolve them meanwhile.  A long list is
-//    matched by the whole grid (grid barriers between the phases of a round), and everything is
-//    resolved after the last round.
-//  - Each round: every live pair offers its key to both particles (atomic min), then its
-//    (id_a, id_b) among equal keys; a pair that is the minimum at both particles is accepted;
-//    pairs touching an accepted particle die, the rest stay live.  The pairs accepted in the
-//    rounds are resolved after the last round.
+//  - The rounds run on block 0 (block barriers) or, for a long list, on as many blocks as it fills
+//    (their own grid barrier between the phases of a round); the other blocks resolve the trivially
+//    accepted pairs and the decays meanwhile, and the pairs accepted in the rounds follow them.
+//  - Each round: every live pair offers its key to both particles (atomic min), FP64 keys then their
+//    (id_a, id_b) among equal keys; a pair that is the minimum at both particles is accepted; pairs
+//    touching an accepted particle die, the rest stay live.
 template <class T>
 __device__ __forceinline__ void ph_match_resolve(
     const DevParams* Pp, DevCtl* ctl, const RepDev* reps,
@@ -1692,7 +1685,7 @@ __device__ __forceinline__ void ph_match_resolve(
     typename V4<T>::type* x1, const uint32_t* id, uint32_t* status,
     typename V4<T>::type* prodpos, uint32_t* deg, uint32_t cap_pairs,
     uint32_t* rep_cons, uint32_t* rep_prod, RepX* repx,
-    ConflictRec* crec, AngJob* jobs, uint32_t job_cap) {
+    ConflictRec* crec, AngJob* jobs, uint32_t job_cap, uint2* events) {
   __shared__ unsigned long long acc_s;
   __shared__ uint32_t live_s;
   const DevParams& P = *Pp;
@@ -1703,7 +1696,9 @@ __device__ __forceinline__ void ph_match_resolve(
     deg[fired[e].ia] = 0u;
     deg[fired[e].ib] = 0u;
   }
-  if (ctl->status) return;
+  if (ctl->status) {
+      return;
+  }
   // n_accept holds the trivially accepted pairs only: the rounds count theirs in n_round_acc, so
   // every block reads the same n_triv whenever it starts
   const uint32_t nc = ctl->n_conflict, n_triv = ctl->n_accept, nd = ctl->n_decay, step = ctl->step;
@@ -1714,34 +1709,37 @@ __device__ __forceinline__ void ph_match_resolve(
   const bool lead = !by_warp || (threadIdx.x & 31) == 0;
   const uint32_t wpb = blockDim.x >> 5, wid = threadIdx.x >> 5;
   const bool multi = nc > (by_warp ? 0u : P.match_single_max) && gridDim.x > 1;
+  // blocks that run the rounds: block 0 for a short list, one per 256 pairs for a long one (at most three
+  // quarters of the grid); the others resolve the trivially accepted pairs and the decays, which involve
+  // no conflict pair, meanwhile.  (With the whole grid in the rounds and everything resolved after them,
+  // 15 000 conflict pairs and 26 000 resolutions of a crowded 2D box took 82 us.)
+  uint32_t nrb = nc > 0 && gridDim.x > 1 ? 1u : 0u;
+  if (multi) nrb = by_warp ? gridDim.x : min((nc + blockDim.x - 1) / blockDim.x, gridDim.x - gridDim.x / 4);
   unsigned long long n_react = 0, n_res = 0, n_near = 0, n_rec = 0;
-  if (!multi) {
-    // block 0 runs the (short) rounds alone, the other blocks resolve meanwhile
-    const bool skip0 = gridDim.x > 1 && nc > 0;
-    const uint32_t nblk = skip0 ? gridDim.x - 1 : gridDim.x;
-    if (!(skip0 && blockIdx.x == 0)) {
-      const uint32_t b = skip0 ? blockIdx.x - 1 : blockIdx.x;
-      const uint32_t q0 = by_warp ? wid * nblk + b : b * blockDim.x + threadIdx.x;
-      for (uint32_t q = q0; q < n_triv + nd; q += nblk * (by_warp ? wpb : blockDim.x)) {
-        const bool pair = q < n_triv;
-        resolve_item<T>(P, reps, fired, fstate, pair, pair ? accepted[q] : decay_list[q - n_triv], step, x0, x1, id,
-                        status, prodpos, rep_cons, rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap, lead);
-      }
+  if (blockIdx.x >= nrb) {
+    const uint32_t nblk = gridDim.x - nrb, b = blockIdx.x - nrb;
+    const uint32_t q0 = by_warp ? wid * nblk + b : b * blockDim.x + threadIdx.x;
+    for (uint32_t q = q0; q < n_triv + nd; q += nblk * (by_warp ? wpb : blockDim.x)) {
+      const bool pair = q < n_triv;
+      resolve_item<T>(P, reps, fired, fstate, pair, pair ? accepted[q] : decay_list[q - n_triv], step, x0, x1, id,
+                      status, prodpos, rep_cons, rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap, events, lead);
     }
   }
   if (nc > 0 && !multi && nc <= min(P.match_smem_max, (uint32_t)kMatchSmemPairs) && blockIdx.x == 0) {
     // short list: block 0 matches in shared memory, then resolves the pairs it accepted
+    if (sizeof(T) == 4)
+      for (uint32_t q = threadIdx.x; q < nc; q += blockDim.x) best_key[crec[q].ia] = best_key[crec[q].ib] = ~0ull;
     if (match_rounds_smem(P, ctl, fired, fstate, matched, conflict, accepted, nc, n_triv)) {
       const uint32_t n_acc = n_triv + *(volatile uint32_t*)&ctl->n_round_acc;
       for (uint32_t q = n_triv + (by_warp ? wid : threadIdx.x); q < n_acc; q += by_warp ? wpb : blockDim.x)
         resolve_item<T>(P, reps, fired, fstate, true, accepted[q], step, x0, x1, id, status, prodpos, rep_cons,
-                        rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap, lead);
+                        rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap, events, lead);
     }
-  } else if (nc > 0 && (multi || blockIdx.x == 0)) {
-    const uint32_t nthr = multi ? gridDim.x * blockDim.x : blockDim.x;
+  } else if (nc > 0 && (multi ? blockIdx.x < nrb : blockIdx.x == 0)) {
+    const uint32_t nthr = multi ? nrb * blockDim.x : blockDim.x;
     const uint32_t tid = multi ? blockIdx.x * blockDim.x + threadIdx.x : threadIdx.x;
     auto sync = [&]() -> bool {
-      if (multi) return grid_barrier(ctl);
+      if (multi) return grid_barrier(ctl, true, &ctl->bar2_count, &ctl->bar2_gen, nrb);
       __syncthreads();
       return true;
     };
@@ -1750,27 +1748,72 @@ __device__ __forceinline__ void ph_match_resolve(
       ctl->live[0] = 0u;
       ctl->live[1] = 0u;
     }
-    // FP32 keys (mixed step) fit one 64-bit word with the partner's id: at a shared particle the
-    // order (key, partner id) is the order (key, id_a, id_b) of its pairs, so the minimum takes
-    // one atomic per endpoint; FP64 keys take the key and then the (id_a, id_b) minimum
-    const bool packed = P.precision == RD_MIXED;
+    auto accept = [&](uint32_t q, const ConflictRec& c) {
+      matched[c.ia] = (int32_t)c.ib;
+      matched[c.ib] = (int32_t)c.ia;
+      fstate[c.e] = (fstate[c.e] & ~3u) | FS_ACCEPTED;
+      crec[q].st = FS_ACCEPTED;
+      accepted[n_triv + atomicAdd(&ctl->n_round_acc, 1u)] = c.e;
+      atomicAdd(&acc_s, 1ull);
+    };
     int rounds = 0;
-    bool ok = sync();
-    while (ok) {
-      for (uint32_t q = tid; q < nc; q += nthr) {
-        const ConflictRec c = crec[q];
-        if (c.st != FS_LIVE) continue;
-        if (packed) {
-          const unsigned long long kb = (unsigned long long)__float_as_uint((float)__longlong_as_double((long long)c.key)) << 32;
-          atomicMin(&best_key[c.ia], kb | (uint32_t)c.pid);
-          atomicMin(&best_key[c.ib], kb | (uint32_t)(c.pid >> 32));
-        } else {
+    bool ok;
+    if constexpr (sizeof(T) == 4) {
+      // two barriers a round: the live pairs offer their keys for the next round to the other minima
+      // array in the phase that empties this round's (the trivial phase made the first offers)
+      __syncthreads();
+      for (;;) {
+        unsigned long long* cur = (rounds & 1) ? best_pid : best_key;
+        unsigned long long* nxt = (rounds & 1) ? best_key : best_pid;
+        for (uint32_t q = tid; q < nc; q += nthr) {
+          const ConflictRec c = crec[q];
+          if (c.st != FS_LIVE) continue;
+          const unsigned long long kb = key_bits_f(c.key);
+          if (cur[c.ia] == (kb | (uint32_t)c.pid) && cur[c.ib] == (kb | (uint32_t)(c.pid >> 32))) accept(q, c);
+        }
+        if (threadIdx.x == 0) live_s = 0u;
+        if (!(ok = sync())) break;
+        const int par = rounds & 1;
+        for (uint32_t q = tid; q < nc; q += nthr) {
+          const ConflictRec c = crec[q];
+          if (c.st == FS_DEAD) continue;
+          cur[c.ia] = ~0ull;
+          cur[c.ib] = ~0ull;
+          if (c.st != FS_LIVE) {
+            if (c.st == FS_ACCEPTED) crec[q].st = FS_DEAD;     // emptied once, not looked at again
+          } else if (matched[c.ia] >= 0 || matched[c.ib] >= 0) {
+            crec[q].st = FS_DEAD;
+            fstate[c.e] = (fstate[c.e] & ~3u) | FS_DEAD;
+          } else {
+            const unsigned long long kb = key_bits_f(c.key);
+            atomicMin(&nxt[c.ia], kb | (uint32_t)c.pid);
+            atomicMin(&nxt[c.ib], kb | (uint32_t)(c.pid >> 32));
+            atomicAdd(&live_s, 1u);
+          }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0 && live_s) atomicAdd(&ctl->live[par], live_s);
+        if (!(ok = sync())) break;
+        ++rounds;
+        if (*(volatile uint32_t*)&ctl->live[par] == 0) break;
+        // the other parity was last read before this round's first barrier
+        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->live[par ^ 1] = 0u;
+        if (rounds >= P.match_max_rounds) {
+          if (blockIdx.x == 0 && threadIdx.x == 0) set_status(ctl, RD_ETIMEOUT);
+          ok = false;
+          break;
+        }
+      }
+    } else {
+      ok = sync();
+      while (ok) {
+        for (uint32_t q = tid; q < nc; q += nthr) {
+          const ConflictRec c = crec[q];
+          if (c.st != FS_LIVE) continue;
           atomicMin(&best_key[c.ia], c.key);
           atomicMin(&best_key[c.ib], c.key);
         }
-      }
-      if (!(ok = sync())) break;
-      if (!packed) {
+        if (!(ok = sync())) break;
         for (uint32_t q = tid; q < nc; q += nthr) {
           const ConflictRec c = crec[q];
           if (c.st != FS_LIVE) continue;
@@ -1778,56 +1821,42 @@ __device__ __forceinline__ void ph_match_resolve(
           if (best_key[c.ib] == c.key) atomicMin(&best_pid[c.ib], c.pid);
         }
         if (!(ok = sync())) break;
-      }
-      for (uint32_t q = tid; q < nc; q += nthr) {
-        const ConflictRec c = crec[q];
-        if (c.st != FS_LIVE) continue;
-        bool win;
-        if (packed) {
-          const unsigned long long kb = (unsigned long long)__float_as_uint((float)__longlong_as_double((long long)c.key)) << 32;
-          win = best_key[c.ia] == (kb | (uint32_t)c.pid) && best_key[c.ib] == (kb | (uint32_t)(c.pid >> 32));
-        } else {
-          win = best_key[c.ia] == c.key && best_key[c.ib] == c.key && best_pid[c.ia] == c.pid &&
-                best_pid[c.ib] == c.pid;
+        for (uint32_t q = tid; q < nc; q += nthr) {
+          const ConflictRec c = crec[q];
+          if (c.st != FS_LIVE) continue;
+          if (best_key[c.ia] == c.key && best_key[c.ib] == c.key && best_pid[c.ia] == c.pid && best_pid[c.ib] == c.pid)
+            accept(q, c);
         }
-        if (win) {
-          matched[c.ia] = (int32_t)c.ib;
-          matched[c.ib] = (int32_t)c.ia;
-          fstate[c.e] = (fstate[c.e] & ~3u) | FS_ACCEPTED;
-          crec[q].st = FS_ACCEPTED;
-          accepted[n_triv + atomicAdd(&ctl->n_round_acc, 1u)] = c.e;
-          atomicAdd(&acc_s, 1ull);
+        if (threadIdx.x == 0) live_s = 0u;
+        if (!(ok = sync())) break;
+        for (uint32_t q = tid; q < nc; q += nthr) {
+          const ConflictRec c = crec[q];
+          if (c.st != FS_LIVE) continue;
+          if (matched[c.ia] >= 0 || matched[c.ib] >= 0) {
+            crec[q].st = FS_DEAD;
+            fstate[c.e] = (fstate[c.e] & ~3u) | FS_DEAD;
+          } else {
+            best_key[c.ia] = ~0ull;
+            best_key[c.ib] = ~0ull;
+            best_pid[c.ia] = ~0ull;
+            best_pid[c.ib] = ~0ull;
+            atomicAdd(&live_s, 1u);
+          }
         }
-      }
-      if (threadIdx.x == 0) live_s = 0u;
-      if (!(ok = sync())) break;
-      for (uint32_t q = tid; q < nc; q += nthr) {
-        const ConflictRec c = crec[q];
-        if (c.st != FS_LIVE) continue;
-        if (matched[c.ia] >= 0 || matched[c.ib] >= 0) {
-          crec[q].st = FS_DEAD;
-          fstate[c.e] = (fstate[c.e] & ~3u) | FS_DEAD;
-        } else {
-          best_key[c.ia] = ~0ull;
-          best_key[c.ib] = ~0ull;
-          best_pid[c.ia] = ~0ull;
-          best_pid[c.ib] = ~0ull;
-          atomicAdd(&live_s, 1u);
+        __syncthreads();
+        const int par = rounds & 1;
+        if (threadIdx.x == 0 && live_s) atomicAdd(&ctl->live[par], live_s);
+        if (!(ok = sync())) break;
+        ++rounds;
+        const uint32_t live = *(volatile uint32_t*)&ctl->live[par];
+        if (live == 0) break;
+        // the other parity was last read before this round's first barrier
+        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->live[par ^ 1] = 0u;
+        if (rounds >= P.match_max_rounds) {
+          if (blockIdx.x == 0 && threadIdx.x == 0) set_status(ctl, RD_ETIMEOUT);
+          ok = false;
+          break;
         }
-      }
-      __syncthreads();
-      const int par = rounds & 1;
-      if (threadIdx.x == 0 && live_s) atomicAdd(&ctl->live[par], live_s);
-      if (!(ok = sync())) break;
-      ++rounds;
-      const uint32_t live = *(volatile uint32_t*)&ctl->live[par];
-      if (live == 0) break;
-      // the other parity was last read before this round's first barrier
-      if (blockIdx.x == 0 && threadIdx.x == 0) ctl->live[par ^ 1] = 0u;
-      if (rounds >= P.match_max_rounds) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) set_status(ctl, RD_ETIMEOUT);
-        ok = false;
-        break;
       }
     }
     if (threadIdx.x == 0) {
@@ -1835,16 +1864,16 @@ __device__ __forceinline__ void ph_match_resolve(
       if (blockIdx.x == 0) atomicAdd(&ctl->stats[RD_STAT_MATCH_ROUNDS], (unsigned long long)rounds);
     }
     // after the last barrier (all blocks of the rounds have passed it): the pairs accepted in the
-    // rounds; with the whole grid in the rounds also the trivially accepted pairs and the decays,
-    // kept out of the barrier-separated phases because a resolution can take long (FP64 2D)
+    // rounds; with the whole grid in the rounds also the trivially accepted pairs and the decays
     if (ok) {
+      const bool all = multi && nrb == gridDim.x;
       const uint32_t n_acc = n_triv + *(volatile uint32_t*)&ctl->n_round_acc;
-      const uint32_t first = multi ? 0u : n_triv, last = multi ? n_acc + nd : n_acc;
+      const uint32_t first = all ? 0u : n_triv, last = all ? n_acc + nd : n_acc;
       const uint32_t q0 = !by_warp ? tid : (multi ? wid * gridDim.x + blockIdx.x : wid);
       for (uint32_t q = first + q0; q < last; q += by_warp ? nthr >> 5 : nthr) {
         const bool pair = q < n_acc;
         resolve_item<T>(P, reps, fired, fstate, pair, pair ? accepted[q] : decay_list[q - n_acc], step, x0, x1, id,
-                        status, prodpos, rep_cons, rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap, lead);
+                        status, prodpos, rep_cons, rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap, events, lead);
       }
     }
   }
@@ -1865,6 +1894,66 @@ __device__ __forceinline__ void ph_match_resolve(
   replica_table(P.n_replicas, reps, rep_cons, rep_prod, repx, ctl);
 }
 
+// The whole matching and resolution of a step with at most one block's threads of fired pairs and
+// decays, by one block: thread q takes pair q, or decay q - nf.  Pairs of degree 1 are accepted at once,
+// the rest go through the shared-memory rounds; then every accepted pair and decay is resolved in one
+// pass.  The chain has no grid barrier and no lists between its stages: 110 pairs 21 -> 14 us.
+template <class T>
+__device__ __forceinline__ void match_resolve_few(
+    const DevParams* Pp, DevCtl* ctl, const RepDev* reps, const FiredPair* fired, uint32_t* fstate, int32_t* matched,
+    uint32_t* conflict, uint32_t* accepted, const uint32_t* decay_list, const typename V4<T>::type* x0,
+    typename V4<T>::type* x1, const uint32_t* id, uint32_t* status, typename V4<T>::type* prodpos, uint32_t* deg,
+    uint32_t cap_pairs, uint32_t* rep_cons, uint32_t* rep_prod, RepX* repx, AngJob* jobs, uint32_t job_cap,
+    uint2* events) {
+  __shared__ uint32_t s_nc;
+  const DevParams& P = *Pp;
+  const uint32_t nf = min(ctl->fired, cap_pairs), nd = ctl->n_decay, step = ctl->step, q = threadIdx.x;
+  const bool aborted = ctl->status != 0;
+  if (q == 0) s_nc = 0u;
+  uint32_t ia = 0, ib = 0, da = 0, db = 0;
+  if (q < nf) {
+    ia = fired[q].ia;
+    ib = fired[q].ib;
+    da = deg[ia];
+    db = deg[ib];
+  }
+  __syncthreads();
+  if (q < nf) {
+    deg[ia] = 0u;
+    deg[ib] = 0u;
+  }
+  if (aborted) return;
+  bool mine = q >= nf && q < nf + nd;      // this thread's item is resolved
+  if (q < nf) {
+    if (da == 1u && db == 1u) {
+      mine = true;
+      matched[ia] = (int32_t)ib;
+      matched[ib] = (int32_t)ia;
+      fstate[q] = (fstate[q] & ~3u) | FS_ACCEPTED;
+    } else {
+      conflict[atomicAdd(&s_nc, 1u)] = q;
+    }
+  }
+  warp_sum_add(&ctl->stats[RD_STAT_MATCHED], q < nf && mine ? 1ull : 0ull);
+  __syncthreads();
+  if (s_nc > 0u) {
+    if (!match_rounds_smem(P, ctl, fired, fstate, matched, conflict, accepted, s_nc, 0u)) return;
+    if (q < nf) mine = (fstate[q] & 3u) == FS_ACCEPTED;
+  }
+  unsigned long long n_react = 0, n_res = 0, n_near = 0, n_rec = 0;
+  if (mine)
+    resolve_item<T>(P, reps, fired, fstate, q < nf, q < nf ? q : decay_list[q - nf], step, x0, x1, id, status, prodpos,
+                    rep_cons, rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap, events, true);
+  if (n_react) atomicAdd(&ctl->stats[RD_STAT_REACTIONS], n_react);
+  if (n_res) atomicAdd(&ctl->stats[RD_STAT_RESAMPLED], n_res);
+  if (n_rec) atomicAdd(&ctl->stats[RD_STAT_RECOMBINED], n_rec);
+  if (n_near) atomicAdd(&ctl->stats[RD_STAT_NEAR_THRESHOLD], n_near);
+  if (P.n_replicas == 1) return;
+  __threadfence();
+  __syncthreads();
+  replica_table(P.n_replicas, reps, rep_cons, rep_prod, repx, ctl);
+}
+
 template <class T>
 __global__ void __launch_bounds__(256, 2) k_match_resolve(
     const DevParams* __restrict__ Pp, DevCtl* __restrict__ ctl, const RepDev* __restrict__ reps,
@@ -1875,15 +1964,23 @@ __global__ void __launch_bounds__(256, 2) k_match_resolve(
     typename V4<T>::type* __restrict__ x1, const uint32_t* __restrict__ id, uint32_t* __restrict__ status,
     typename V4<T>::type* __restrict__ prodpos, uint32_t* __restrict__ deg, uint32_t cap_pairs,
     uint32_t* __restrict__ rep_cons, uint32_t* __restrict__ rep_prod, RepX* __restrict__ repx,
-    ConflictRec* __restrict__ crec, AngJob* __restrict__ jobs, uint32_t job_cap) {
+    ConflictRec* __restrict__ crec, AngJob* __restrict__ jobs, uint32_t job_cap, uint2* __restrict__ events) {
   pdl_enter();
+  // few pairs and decays: block 0 alone, without grid barriers (a thread per item)
+  if (!(sizeof(T) == 8 && Pp->dim == 2) && Pp->match_smem_max >= 256u && Pp->match_single_max > 0u &&
+      ctl->fired + ctl->n_decay <= blockDim.x) {
+    if (blockIdx.x == 0)
+      match_resolve_few<T>(Pp, ctl, reps, fired, fstate, matched, conflict, accepted, decay_list, x0, x1, id, status,
+                           prodpos, deg, cap_pairs, rep_cons, rep_prod, repx, jobs, job_cap, events);
+    return;
+  }
   // the degree-1 pairs accepted and the rest listed as conflicts first, then (every block past the
   // barrier) the rounds and the resolution: one launch for both stages
   ph_match_trivial(ctl, fired, fstate, deg, matched, conflict, accepted, best_key, best_pid,
-                   cap_pairs, crec, blockIdx.x, gridDim.x);
+                   cap_pairs, crec, sizeof(T) == 4, blockIdx.x, gridDim.x);
   if (!grid_barrier(ctl, false)) return;
   ph_match_resolve<T>(Pp, ctl, reps, fired, fstate, matched, conflict, accepted, best_key, best_pid, decay_list, x0,
-                      x1, id, status, prodpos, deg, cap_pairs, rep_cons, rep_prod, repx, crec, jobs, job_cap);
+                      x1, id, status, prodpos, deg, cap_pairs, rep_cons, rep_prod, repx, crec, jobs, job_cap, events);
 }
 
 // Places the two particles of angle job j along dir (the new separation direction).
@@ -1974,17 +2071,21 @@ __global__ void __launch_bounds__(256, 2) k_angles(const DevParams* __restrict__
   ph_angles<T>(Pp, ctl, reps, jobs, job_cap, x1, prodpos, blockIdx.x, gridDim.x);
 }
 
+// Count of a (replica, species) key: atomically up or down by one.  Only particles that leave or join
+// are counted; the counts carry over from step to step.
+__device__ __forceinline__ void count_event(uint32_t wb, int ns, bool up, unsigned long long* counts, int32_t* s_tot) {
+  const unsigned long long one = 1ull;
+  atomicAdd(&counts[(size_t)(wb >> 8) * ns + (wb & 0xFFu)], up ? one : ~0ull);
+  atomicAdd(&s_tot[wb & 0xFFu], up ? 1 : -1);
+}
+
 // Per-warp aggregated count: lanes holding the same (replica, species) key add once.  Called by all
 // 32 lanes of a converged warp; key kNoKey is skipped.
 constexpr uint32_t kNoKey = 0xFFFFFFFFu;
-__device__ __forceinline__ void count_key(uint32_t key, bool smem, uint32_t* hist, unsigned long long* counts) {
+__device__ __forceinline__ void count_key(uint32_t key, unsigned long long* counts) {
   const unsigned peers = __match_any_sync(0xFFFFFFFFu, key);
-  if (key != kNoKey && (int)(threadIdx.x & 31) == __ffs(peers) - 1) {
-    if (smem)
-      atomicAdd(&hist[key], (uint32_t)__popc(peers));
-    else
-      atomicAdd(&counts[key], (unsigned long long)__popc(peers));
-  }
+  if (key != kNoKey && (int)(threadIdx.x & 31) == __ffs(peers) - 1)
+    atomicAdd(&counts[key], (unsigned long long)__popc(peers));
 }
 
 // Species totals over all replicas of the (replica, species) counts, by one whole block.
@@ -2006,40 +2107,55 @@ __device__ __forceinline__ void species_totals(const unsigned long long* counts,
 }
 
 // ================================================================================================
-// K7: compaction, one pass.  Tiles of 2048 particles scan (survivor, products) counts
-// with a decoupled look-back, then place their own particles: survivors keep their order inside
-// their replica, products follow the replica's survivors in owner order with ids next_id + rank
-// (the per-replica offsets come from the table built at the end of the resolution).  An error
-// latched during the step, or a particle count above capacity, turns this into a copy of the
-// unchanged state.  The last block to finish commits the step.
+// K7: compaction, one pass.  Tiles of 2048 particles: survivors keep their order inside their replica,
+// products follow the replica's survivors in owner order with ids next_id + rank (the per-replica
+// offsets come from the table built at the end of the resolution).  A particle's place follows from the
+// number of consumed particles and of products before it.  With up to kMaxEvents consumed particles
+// every tile takes these from the step's event list (a count of the events before the tile, and the few
+// inside it), so that no tile waits for another; with more, the tiles scan the status words with a
+// decoupled look-back.  An error latched during the step, or a particle count above capacity, turns this
+// into a copy of the unchanged state.  The last block to finish commits the step.
 // ================================================================================================
-constexpr int kCompactTile = 2048;   // particles per tile (the look-back buffers are sized for it)
-
 template <class T, int kCompactThreads>
 __device__ __forceinline__ void ph_compact(const DevParams* Pp, DevCtl* ctl,
                           RepDev* reps, const RepX* repx,
                           uint32_t* rep_cons, uint32_t* rep_prod,
                           const typename V4<T>::type* x0,
                           const typename V4<T>::type* x1, const uint32_t* id,
-                          const uint32_t* status, const typename V4<T>::type* prodpos,
+                          const uint32_t* status, const typename V4<T>::type* prodpos, const uint2* events,
                           unsigned long long* agg, unsigned long long* incl,
                           uint32_t* flag, typename V4<T>::type* xo,
-                          uint32_t* ido, unsigned long long* counts, int n_counts,
+                          uint32_t* ido, unsigned long long* counts,
                           long long* history, int history_len,
-                          uint32_t* hist /* n_counts entries when n_counts <= kSmemCounts */,
-                          unsigned long long* s_pre /* kCompactTile entries */,
+                          unsigned long long* s_pre /* kCompactTile entries */, const uint32_t cap,
+                          const uint32_t bid, const uint32_t nblk,
                           const int stamp_phase = -1) {
   constexpr int kTile = kCompactTile, kCompactItems = kCompactTile / kCompactThreads;
+  constexpr int kPasses = kCompactItems;
   __shared__ unsigned long long sm[32];
   __shared__ uint32_t s_tile;
   __shared__ unsigned long long s_prefix;
   __shared__ bool s_last;
+  __shared__ int32_t s_tot[kMaxSpecies];
+  __shared__ uint32_t s_before[2], s_inside;
   const DevParams& P = *Pp;
+  // the first tile's loads go out beside those of the control block (four passes at most)
+  constexpr int kAhead = kPasses < 4 ? kPasses : 4;
+  typename V4<T>::type q[kAhead];
+  uint32_t idv[kAhead];
+  auto load_passes = [&](const int64_t t0, const int first, const uint32_t end) {
+#pragma unroll
+    for (int ps = 0; ps < kAhead; ++ps) {
+      const int64_t i = t0 + threadIdx.x + (first + ps) * kCompactThreads;
+      if (i < (int64_t)end) {
+        q[ps] = x1[i];
+        idv[ps] = id[i];
+      }
+    }
+  };
+  load_passes((int64_t)bid * kTile, 0, cap);
   const int ns = P.n_species;
-  const bool use_smem = n_counts <= kSmemCounts;
-  if (use_smem)
-    for (int k = threadIdx.x; k < n_counts; k += blockDim.x) hist[k] = 0u;
-  const uint32_t n = ctl->n;
+  const uint32_t n = ctl->n, n_ev = ctl->n_ev;
   // a single replica: its placement follows from the step's tallies directly
   const bool one = P.n_replicas == 1;
   RepX rx1 = {0u, 0u, 0u, 0u};
@@ -2050,116 +2166,158 @@ __device__ __forceinline__ void ph_compact(const DevParams* Pp, DevCtl* ctl,
   }
   const uint32_t n_new = one ? rx1.surv + rx1.prod : ctl->n_new;
   const bool fail = ctl->status != 0 || (unsigned long long)n_new > (unsigned long long)P.cap_particles;
+  const bool few = !fail && n_ev <= kMaxEvents;
   const uint32_t ntiles = (uint32_t)(((int64_t)n + kTile - 1) / kTile);
-  auto key_of = [&](uint32_t wb) { return (wb >> 8) * ns + (wb & 0xFFu); };
-  // tiles by ticket, so that every tile's predecessors are taken before it (look-back order)
-  for (;;) {
-    __syncthreads();
-    if (threadIdx.x == 0) s_tile = atomicAdd(&ctl->tile_ctr[1], 1u);
-    __syncthreads();
-    const uint32_t tile = s_tile;
-    if (tile >= ntiles) break;
-    const int64_t t0 = (int64_t)tile * kTile;
-    // with at most two placement passes per thread, the placement's loads go out before the scan,
-    // so that their latency overlaps the scan and the look-back (more passes' worth of registers
-    // cost occupancy: 512-thread tiles with four early passes ran at half the speed)
-    constexpr int kPasses = kTile / kCompactThreads;
-    constexpr bool kEarly = kPasses <= 2;
-    typename V4<T>::type q_r[kEarly ? kPasses : 1];
-    uint32_t st_r[kEarly ? kPasses : 1], id_r[kEarly ? kPasses : 1];
-    if constexpr (kEarly) {
+  if (threadIdx.x < kMaxSpecies) s_tot[threadIdx.x] = 0;
+  // the products of owner i, P_i products before it
+  auto place_products = [&](uint32_t i, uint32_t np, uint32_t P_i, const RepX& rx, uint32_t r) {
+    for (uint32_t k = 0; k < np; ++k) {
+      const uint32_t o = rx.s_end + P_i + k;
+      const auto pp = prodpos[2 * (size_t)i + k];
+      xo[o] = pp;
+      ido[o] = reps[r].next_id + (P_i - rx.p_beg) + k;
+      if (!few) count_event(w_bits(pp.w), ns, true, counts, s_tot);
+    }
+  };
+  if (few) {
+    uint32_t* inside = reinterpret_cast<uint32_t*>(s_pre);
+    for (uint32_t tile = bid; tile < ntiles; tile += nblk) {
+      const int64_t t0 = (int64_t)tile * kTile;
+      __syncthreads();
+      if (threadIdx.x == 0) s_before[0] = s_before[1] = s_inside = 0u;
+      __syncthreads();
+      if (tile != bid) load_passes(t0, 0, n);
+      uint32_t cb = 0, pb = 0;
+      for (uint32_t e = threadIdx.x; e < n_ev; e += kCompactThreads) {
+        const uint2 v = events[e];
+        if ((int64_t)v.x < t0) {
+          ++cb;
+          pb += v.y;
+        } else if ((int64_t)v.x < t0 + kTile) {
+          inside[atomicAdd(&s_inside, 1u)] = ((uint32_t)(v.x - t0) << 2) | v.y;
+        }
+      }
+      cb = __reduce_add_sync(0xFFFFFFFFu, cb);
+      pb = __reduce_add_sync(0xFFFFFFFFu, pb);
+      if ((threadIdx.x & 31) == 0 && cb) {
+        atomicAdd(&s_before[0], cb);
+        atomicAdd(&s_before[1], pb);
+      }
+      __syncthreads();
+      const uint32_t m = s_inside, c0 = s_before[0], p0 = s_before[1];
+#pragma unroll
+      for (int p0s = 0; p0s < kPasses; p0s += kAhead) {
+        if (p0s > 0) load_passes(t0, p0s, n);
+#pragma unroll
+        for (int ps = 0; ps < kAhead; ++ps) {
+          const uint32_t j = threadIdx.x + (p0s + ps) * kCompactThreads;
+          const int64_t i = t0 + j;
+          if (i >= (int64_t)n) continue;
+          uint32_t S_i = (uint32_t)i - c0, P_i = p0, np = 0;
+          bool gone = false;
+          for (uint32_t e = 0; e < m; ++e) {
+            const uint32_t v = inside[e], l = v >> 2;
+            S_i -= l < j;
+            P_i += l < j ? v & 3u : 0u;
+            if (l == j) {
+              gone = true;
+              np = v & 3u;
+            }
+          }
+          const uint32_t r = w_bits(q[ps].w) >> 8;
+          const RepX rx = one ? rx1 : repx[r];
+          if (!gone) {
+            xo[S_i + rx.p_beg] = q[ps];
+            ido[S_i + rx.p_beg] = idv[ps];
+          } else {
+            place_products((uint32_t)i, np, P_i, rx, r);
+          }
+        }
+      }
+    }
+  } else {
+    // tiles by ticket, so that every tile's predecessors are taken before it (look-back order)
+    for (;;) {
+      __syncthreads();
+      if (threadIdx.x == 0) s_tile = atomicAdd(&ctl->tile_ctr[1], 1u);
+      __syncthreads();
+      const uint32_t tile = s_tile;
+      if (tile >= ntiles) break;
+      const int64_t t0 = (int64_t)tile * kTile;
+      if (!fail) {
+        // blocked arrangement for the scan: each thread owns kCompactItems consecutive particles
+        const int64_t base = t0 + (int64_t)threadIdx.x * kCompactItems;
+        unsigned long long v[kCompactItems], ex[kCompactItems], run = 0;
+        if constexpr (kCompactItems == 8) {
+          LoadCompact{status}.load8(base, n, v);
+        } else {
+#pragma unroll
+          for (int k = 0; k < kCompactItems; ++k) v[k] = base + k < (int64_t)n ? LoadCompact::conv(__ldcg(status + base + k)) : 0ull;
+        }
+#pragma unroll
+        for (int k = 0; k < kCompactItems; ++k) {
+          ex[k] = run;
+          run += v[k];
+        }
+        unsigned long long tot;
+        const unsigned long long toff = block_exclusive_scan<unsigned long long, int>(run, sm, tot);
+        if (threadIdx.x < 32) {
+          const uint32_t epoch = (ctl->epoch * 2u + 1u) & 0x3FFFFFFFu;
+          const unsigned long long prefix = tile_lookback<unsigned long long>(tot, tile, epoch, agg, incl, flag, ctl);
+          if (threadIdx.x == 0) s_prefix = prefix;
+        }
+        __syncthreads();
+        const unsigned long long pre = s_prefix + toff;
+#pragma unroll
+        for (int k = 0; k < kCompactItems; ++k) s_pre[threadIdx.x * kCompactItems + k] = pre + ex[k];
+        __syncthreads();
+      }
+      // striped placement (coalesced), one particle per thread per pass
 #pragma unroll
       for (int ps = 0; ps < kPasses; ++ps) {
-        const int64_t i = t0 + threadIdx.x + ps * kCompactThreads;
-        if (i < (int64_t)n) {
-          q_r[ps] = fail ? x0[i] : x1[i];
-          st_r[ps] = fail ? 0u : status[i];
-          id_r[ps] = id[i];
-        }
-      }
-    }
-    if (!fail) {
-      // blocked arrangement for the scan: each thread owns kCompactItems consecutive particles
-      const int64_t base = t0 + (int64_t)threadIdx.x * kCompactItems;
-      unsigned long long v[kCompactItems], ex[kCompactItems], run = 0;
-      if constexpr (kCompactItems == 8) {
-        LoadCompact{status}.load8(base, n, v);
-      } else {
-#pragma unroll
-        for (int k = 0; k < kCompactItems; ++k) v[k] = base + k < (int64_t)n ? LoadCompact::conv(__ldcg(status + base + k)) : 0ull;
-      }
-#pragma unroll
-      for (int k = 0; k < kCompactItems; ++k) {
-        ex[k] = run;
-        run += v[k];
-      }
-      unsigned long long tot;
-      const unsigned long long toff = block_exclusive_scan<unsigned long long, int>(run, sm, tot);
-      if (threadIdx.x < 32) {
-        const uint32_t epoch = (ctl->epoch * 2u + 1u) & 0x3FFFFFFFu;
-        const unsigned long long prefix = tile_lookback<unsigned long long>(tot, tile, epoch, agg, incl, flag, ctl);
-        if (threadIdx.x == 0) s_prefix = prefix;
-      }
-      __syncthreads();
-      const unsigned long long pre = s_prefix + toff;
-#pragma unroll
-      for (int k = 0; k < kCompactItems; ++k) s_pre[threadIdx.x * kCompactItems + k] = pre + ex[k];
-      __syncthreads();
-    }
-    // striped placement (coalesced), one particle per thread per pass, warp-converged counting
-#pragma unroll
-    for (int ps = 0; ps < kPasses; ++ps) {
-      const int j = threadIdx.x + ps * kCompactThreads;
-      const int64_t i = t0 + j;
-      uint32_t k0 = kNoKey, k1 = kNoKey, k2 = kNoKey;
-      if (i < (int64_t)n) {
+        const int j = threadIdx.x + ps * kCompactThreads;
+        const int64_t i = t0 + j;
+        if (i >= (int64_t)n) continue;
         if (fail) {
-          const auto q0 = kEarly ? q_r[kEarly ? ps : 0] : x0[i];
-          xo[i] = q0;
-          ido[i] = kEarly ? id_r[kEarly ? ps : 0] : id[i];
-          k0 = key_of(w_bits(q0.w));
-        } else {
-          const unsigned long long e = s_pre[j];
-          const uint32_t S_i = (uint32_t)(e >> 32), P_i = (uint32_t)e;
-          const uint32_t st = kEarly ? st_r[kEarly ? ps : 0] : status[i];
-          const auto q = kEarly ? q_r[kEarly ? ps : 0] : x1[i];
-          const uint32_t wb = w_bits(q.w);
-          const uint32_t r = wb >> 8;
-          const RepX rx = one ? rx1 : repx[r];
-          if (!(st & ST_CONSUMED)) {
-            const uint32_t o = S_i + rx.p_beg;
-            xo[o] = q;
-            ido[o] = kEarly ? id_r[kEarly ? ps : 0] : id[i];
-            k0 = key_of(wb);
-          }
-          const uint32_t np = (st >> ST_NPROD_SHIFT) & 3u;
-          for (uint32_t k = 0; k < np; ++k) {
-            const uint32_t o = rx.s_end + P_i + k;
-            const auto pp = prodpos[2 * (size_t)i + k];
-            xo[o] = pp;
-            ido[o] = reps[r].next_id + (P_i - rx.p_beg) + k;
-            (k == 0 ? k1 : k2) = key_of(w_bits(pp.w));
-          }
+          xo[i] = x0[i];
+          ido[i] = id[i];
+          continue;
         }
+        const unsigned long long e = s_pre[j];
+        const uint32_t S_i = (uint32_t)(e >> 32), P_i = (uint32_t)e;
+        const uint32_t st = status[i];
+        const auto q = x1[i];
+        const uint32_t wb = w_bits(q.w), r = wb >> 8;
+        const RepX rx = one ? rx1 : repx[r];
+        if (!(st & ST_CONSUMED)) {
+          const uint32_t o = S_i + rx.p_beg;
+          xo[o] = q;
+          ido[o] = id[i];
+        } else {
+          count_event(wb, ns, false, counts, s_tot);
+        }
+        place_products((uint32_t)i, (st >> ST_NPROD_SHIFT) & 3u, P_i, rx, r);
       }
-      count_key(k0, use_smem, hist, counts);
-      if (__any_sync(0xFFFFFFFFu, k1 != kNoKey)) count_key(k1, use_smem, hist, counts);
-      if (__any_sync(0xFFFFFFFFu, k2 != kNoKey)) count_key(k2, use_smem, hist, counts);
     }
-  }
-  if (use_smem) {
     __syncthreads();
-    for (int k = threadIdx.x; k < n_counts; k += blockDim.x)
-      if (hist[k]) atomicAdd(&counts[k], (unsigned long long)hist[k]);
+    if (threadIdx.x < (unsigned)ns && s_tot[threadIdx.x]) atomicAdd((unsigned long long*)&ctl->tot[threadIdx.x], (unsigned long long)(long long)s_tot[threadIdx.x]);
+    __threadfence();
   }
+  // the last block to finish commits the step: counts, replica segments, ids, particle count, step, time
+  // (with the event list it reads nothing that another block wrote, so no fence precedes its arrival)
   __syncthreads();
-  // the last block to finish commits the step: replica segments, ids, count, step, time
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&ctl->done_blocks, 1u) == gridDim.x - 1;
+  if (threadIdx.x == 0) s_last = atomicAdd(&ctl->done_blocks, 1u) == nblk - 1;
   __syncthreads();
   if (!s_last) return;
-  __threadfence();
+  if (few) {
+    for (uint32_t e = threadIdx.x; e < n_ev; e += blockDim.x) {
+      const uint2 v = events[e];
+      count_event(w_bits(x0[v.x].w), ns, false, counts, s_tot);
+      for (uint32_t k = 0; k < v.y; ++k) count_event(w_bits(prodpos[2 * (size_t)v.x + k].w), ns, true, counts, s_tot);
+    }
+  } else {
+    __threadfence();
+  }
   for (int r = threadIdx.x; r < P.n_replicas; r += blockDim.x) {
     if (!fail) {
       const RepX rx = one ? rx1 : repx[r];
@@ -2171,9 +2329,13 @@ __device__ __forceinline__ void ph_compact(const DevParams* Pp, DevCtl* ctl,
     rep_cons[r] = 0u;
     rep_prod[r] = 0u;
   }
+  __syncthreads();
   // per-step totals over replicas of every species (ring buffer indexed by the new step)
-  if (!fail && history_len > 0)
-    species_totals(counts, P.n_replicas, ns, history + (size_t)((ctl->step + 1u) % (uint32_t)history_len) * ns);
+  if (!fail && threadIdx.x < (unsigned)ns) {
+    const long long t = *(volatile long long*)&ctl->tot[threadIdx.x] + (few ? (long long)s_tot[threadIdx.x] : 0ll);
+    ctl->tot[threadIdx.x] = t;
+    if (history_len > 0) history[(size_t)((ctl->step + 1u) % (uint32_t)history_len) * ns + threadIdx.x] = t;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     if (stamp_phase >= 0) {
@@ -2200,6 +2362,7 @@ __device__ __forceinline__ void ph_compact(const DevParams* Pp, DevCtl* ctl,
     ctl->n_accept = 0;
     ctl->n_round_acc = 0;
     ctl->n_ang = 0;
+    ctl->n_ev = 0;
     ctl->n_decay = 0;
     ctl->done_blocks = 0;
     ctl->done_res = 0;
@@ -2213,15 +2376,15 @@ __global__ void __launch_bounds__(kCompactThreads) k_compact(const DevParams* __
                           const typename V4<T>::type* __restrict__ x0,
                           const typename V4<T>::type* __restrict__ x1, const uint32_t* __restrict__ id,
                           const uint32_t* __restrict__ status, const typename V4<T>::type* __restrict__ prodpos,
+                          const uint2* __restrict__ events,
                           unsigned long long* __restrict__ agg, unsigned long long* __restrict__ incl,
                           uint32_t* __restrict__ flag, typename V4<T>::type* __restrict__ xo,
-                          uint32_t* __restrict__ ido, unsigned long long* __restrict__ counts, int n_counts,
-                          long long* __restrict__ history, int history_len) {
+                          uint32_t* __restrict__ ido, unsigned long long* __restrict__ counts,
+                          long long* __restrict__ history, int history_len, const uint32_t cap) {
   pdl_enter();
-  extern __shared__ uint32_t hist[];   // n_counts entries when n_counts <= kSmemCounts
   __shared__ unsigned long long s_pre[kCompactTile];
-  ph_compact<T, kCompactThreads>(Pp, ctl, reps, repx, rep_cons, rep_prod, x0, x1, id, status, prodpos, agg, incl,
-                                 flag, xo, ido, counts, n_counts, history, history_len, hist, s_pre);
+  ph_compact<T, kCompactThreads>(Pp, ctl, reps, repx, rep_cons, rep_prod, x0, x1, id, status, prodpos, events, agg, incl,
+                                 flag, xo, ido, counts, history, history_len, s_pre, cap, blockIdx.x, gridDim.x);
 }
 
 // ================================================================================================
@@ -2274,7 +2437,7 @@ __global__ void k_count(const DevParams* __restrict__ Pp, const DevCtl* __restri
       const uint32_t wb = w_bits(x[i].w);
       key = (wb >> 8) * Pp->n_species + (wb & 0xFFu);
     }
-    count_key(key, false, nullptr, counts);
+    count_key(key, counts);
   }
 }
 
@@ -2576,12 +2739,10 @@ __global__ void __launch_bounds__(256, 2) k_step_fused(const StepLaunch L, const
     uint32_t* ido = odd ? L.id_cur : L.id_next;
     V* x0s = L.x0d ? (V*)L.x0d : x0;
     V* x1 = (V*)L.x1;
-    V* sx0 = (V*)L.sx0;
-    V* sx1 = (V*)L.sx1;
     V* prod = (V*)L.prodpos;
     phase_stamp(ctl, 0);
-    ph_prepare<T>(L.P, ctl, L.reps, x0, id0, x1, L.status, L.cell_of, L.slot, L.cell_count, L.decay_list, L.counts,
-                  L.n_counts, L.x0d ? x0s : (V*)nullptr, blockIdx.x, gridDim.x);
+    ph_prepare<T>(L.P, ctl, L.reps, x0, id0, x1, L.status, L.cell_of, L.slot, L.cell_count, L.decay_list,
+                  L.x0d ? x0s : (V*)nullptr, (uint32_t)L.cap_particles, blockIdx.x, gridDim.x);
     if (!grid_barrier(ctl, false)) return;
     phase_stamp(ctl, 1);
     while (ph_scan_tile<uint32_t, LoadCellCount>(LoadCellCount{L.cell_count}, L.total_cells, nullptr, L.cell_start,
@@ -2589,21 +2750,21 @@ __global__ void __launch_bounds__(256, 2) k_step_fused(const StepLaunch L, const
     }
     if (!grid_barrier(ctl, false)) return;
     phase_stamp(ctl, 2);
-    ph_scatter<T>(ctl, x0s, x1, id0, L.cell_of, L.slot, L.cell_start, sx0, sx1, L.sidx, blockIdx.x, gridDim.x);
+    ph_scatter<T>(L.P, ctl, x0s, L.cell_of, L.slot, L.cell_start, L.rec, (uint32_t)L.cap_particles, blockIdx.x, gridDim.x);
     if (!grid_barrier(ctl, false)) return;
     phase_stamp(ctl, 3);
-    ph_sweep<T, kSplit, kReach>(L.P, ctl, L.reps, sx0, sx1, L.sidx, L.cell_start, L.total_cells, L.fired, L.fstate,
+    ph_sweep<T, kSplit, kReach>(L.P, ctl, L.reps, x0s, x1, id0, L.rec, L.cell_start, L.total_cells, L.fired, L.fstate,
                                 L.deg, L.matched, (uint32_t)L.cap_pairs, split, (uint2(*)[256])dsm, blockIdx.x,
                                 gridDim.x);
     if (!grid_barrier(ctl, false)) return;
     phase_stamp(ctl, 4);
     ph_match_trivial(ctl, L.fired, L.fstate, L.deg, L.matched, L.conflict, L.accepted, L.best_key, L.best_pid,
-                     (uint32_t)L.cap_pairs, L.crec, blockIdx.x, gridDim.x);
+                     (uint32_t)L.cap_pairs, L.crec, sizeof(T) == 4, blockIdx.x, gridDim.x);
     if (!grid_barrier(ctl, false)) return;
     phase_stamp(ctl, 5);
     ph_match_resolve<T>(L.P, ctl, L.reps, L.fired, L.fstate, L.matched, L.conflict, L.accepted, L.best_key,
                         L.best_pid, L.decay_list, x0s, x1, id0, L.status, prod, L.deg, (uint32_t)L.cap_pairs,
-                        L.rep_cons, L.rep_prod, L.repx, L.crec, L.ang_jobs, L.ang_cap);
+                        L.rep_cons, L.rep_prod, L.repx, L.crec, L.ang_jobs, L.ang_cap, L.events);
     if (!grid_barrier(ctl, false)) return;
     phase_stamp(ctl, 6);
     if (L.angles) {
@@ -2612,9 +2773,9 @@ __global__ void __launch_bounds__(256, 2) k_step_fused(const StepLaunch L, const
     }
     phase_stamp(ctl, 7);
     ph_compact<T, 256>(L.P, ctl, L.reps, (const RepX*)L.repx, L.rep_cons, L.rep_prod, x0, x1, id0, L.status, prod,
-                       L.agg64, L.incl64, L.flags + L.flag_stride, xo, ido, L.counts, L.n_counts, L.history,
-                       L.history_len, (uint32_t*)(dsm + sizeof(unsigned long long) * kCompactTile),
-                       (unsigned long long*)dsm, 7);
+                       (const uint2*)L.events, L.agg64, L.incl64, L.flags + L.flag_stride, xo, ido, L.counts, L.history,
+                       L.history_len, (unsigned long long*)dsm, (uint32_t)L.cap_particles, blockIdx.x,
+                       gridDim.x, 7);
     if (st + 1 < nsteps) {
       // the next step starts from the committed state; after an error the state is kept and the
       // remaining steps are not taken
@@ -2624,9 +2785,8 @@ __global__ void __launch_bounds__(256, 2) k_step_fused(const StepLaunch L, const
   }
 }
 
-static size_t fused_smem_bytes(const StepLaunch& L) {
-  const size_t hist = L.n_counts <= kSmemCounts ? (size_t)L.n_counts * 4 : 0;
-  return std::max(kFusedSmemSweep, sizeof(unsigned long long) * kCompactTile + hist);
+static size_t fused_smem_bytes() {
+  return std::max(kFusedSmemSweep, sizeof(unsigned long long) * kCompactTile);
 }
 
 template <class T>
@@ -2645,10 +2805,10 @@ int fused_grid_size(const StepLaunch& L, int device_sms) {
   int per_sm = 0;
   // static (conflict rounds, ~28 KB) plus dynamic shared memory exceeds the default 48 KB per
   // block: opt in to the larger dynamic size (per kernel, per device)
-  if (cudaFuncSetAttribute(fused_kernel(L), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fused_smem_bytes(L)) !=
+  if (cudaFuncSetAttribute(fused_kernel(L), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fused_smem_bytes()) !=
       cudaSuccess)
     return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fused_kernel(L), 256, fused_smem_bytes(L)) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fused_kernel(L), 256, fused_smem_bytes()) !=
       cudaSuccess)
     return 0;
   per_sm = std::min(per_sm, 2);
@@ -2659,7 +2819,7 @@ void launch_fused_steps(const StepLaunch& L, int nsteps, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)std::max(L.fused_grid, 1));
   cfg.blockDim = dim3(256u);
-  cfg.dynamicSmemBytes = fused_smem_bytes(L);
+  cfg.dynamicSmemBytes = fused_smem_bytes();
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
@@ -2726,6 +2886,16 @@ int match_grid_size(int device_sms) {
   return per_sm >= 1 ? device_sms * per_sm : 1;
 }
 
+// The matching launch of a step.
+template <class T>
+static void launch_match(const StepLaunch& L, bool pdl, cudaStream_t s) {
+  using V = typename V4<T>::type;
+  launch_coop(pdl, k_match_resolve<T>, L.match_grid > 0 ? L.match_grid : 1, 256, s, L.P, L.ctl, L.reps, L.fired, L.fstate,
+              L.matched, L.conflict, L.accepted, L.best_key, L.best_pid, L.decay_list,
+              (V*)(L.x0d ? L.x0d : L.x_cur), (V*)L.x1, L.id_cur, L.status, (V*)L.prodpos, L.deg,
+              (uint32_t)L.cap_pairs, L.rep_cons, L.rep_prod, L.repx, L.crec, L.ang_jobs, L.ang_cap, L.events);
+}
+
 template <class T>
 static void step_impl(const StepLaunch& L, cudaStream_t s, KernelTimer* timer) {
   using V = typename V4<T>::type;
@@ -2737,24 +2907,22 @@ static void step_impl(const StepLaunch& L, cudaStream_t s, KernelTimer* timer) {
   V* x0 = (V*)L.x_cur;
   V* xo = (V*)L.x_next;
   V* x1 = (V*)L.x1;
-  V* sx0 = (V*)L.sx0;
-  V* sx1 = (V*)L.sx1;
   V* prod = (V*)L.prodpos;
-  const int64_t tile = 256 * (int64_t)kScanItems;
 
   mark("begin");
   const bool pdl = L.pdl;
   // start-of-step positions of the step proper: drifted copies when there is a drift step
   V* x0s = L.x0d ? (V*)L.x0d : x0;
+  const uint32_t cap = (uint32_t)L.cap_particles;
   launch_k(pdl, k_prepare<T>, Gp, B, 0, s, L.P, L.ctl, L.reps, x0, L.id_cur, x1, L.status, L.cell_of, L.slot,
-           L.cell_count, L.decay_list, L.counts, L.n_counts, L.x0d ? x0s : (V*)nullptr);
+           L.cell_count, L.decay_list, L.x0d ? x0s : (V*)nullptr, cap);
   mark("k_prepare");
+  const int64_t tile = 256 * (int64_t)kScanItems;
   const int nbc = (int)((L.total_cells + tile - 1) / tile);
   launch_k(pdl, k_scan1<uint32_t, LoadCellCount>, nbc, 256, 0, s, LoadCellCount{L.cell_count}, L.total_cells,
            (const uint32_t*)nullptr, L.cell_start, L.cell_count, L.agg32, L.incl32, L.flags, L.ctl, 0);
   mark("k_scan_cells");
-  launch_k(pdl, k_scatter_cells<T>, Gp, B, 0, s, L.ctl, x0s, x1, L.id_cur, L.cell_of, L.slot, L.cell_start, sx0,
-           sx1, L.sidx);
+  launch_k(pdl, k_scatter_cells<T>, Gp, B, 0, s, L.P, L.ctl, x0s, L.cell_of, L.slot, L.cell_start, L.rec, cap);
   mark("k_scatter_cells");
   const uint32_t split = L.sweep_split > 1 ? (uint32_t)L.sweep_split : 1u;
   // FP64 in 2D: one-warp blocks, so that the warp-wide p_enc evaluations (the FP64 pipe of an SM is
@@ -2762,17 +2930,15 @@ static void step_impl(const StepLaunch& L, cudaStream_t s, KernelTimer* timer) {
   const int Bs = sizeof(T) == 8 && L.dim == 2 ? 32 : 256;
   const int Gs = grid_for(L.cap_particles * (int64_t)split, Bs, L.max_grid);
   auto sweep = [&](auto kernel) {
-    launch_k(pdl, kernel, Gs, Bs, 0, s, L.P, L.ctl, L.reps, sx0, sx1, L.sidx, L.cell_start, L.total_cells, L.fired,
-             L.fstate, L.deg, L.matched, (uint32_t)L.cap_pairs, split);
+    launch_k(pdl, kernel, Gs, Bs, 0, s, L.P, L.ctl, L.reps, x0s, x1, L.id_cur, L.rec, L.cell_start, L.total_cells,
+             L.fired, L.fstate, L.deg, L.matched, (uint32_t)L.cap_pairs, split);
   };
   if (L.reach == 2)
     split > 1 ? sweep(k_sweep<T, true, 2>) : sweep(k_sweep<T, false, 2>);
   else
     split > 1 ? sweep(k_sweep<T, true, 1>) : sweep(k_sweep<T, false, 1>);
   mark("k_sweep");
-  launch_coop(pdl, k_match_resolve<T>, L.match_grid > 0 ? L.match_grid : 1, 256, s, L.P, L.ctl, L.reps, L.fired, L.fstate,
-              L.matched, L.conflict, L.accepted, L.best_key, L.best_pid, L.decay_list, x0s, x1, L.id_cur, L.status,
-              prod, L.deg, (uint32_t)L.cap_pairs, L.rep_cons, L.rep_prod, L.repx, L.crec, L.ang_jobs, L.ang_cap);
+  launch_match<T>(L, pdl, s);
   mark("k_match_resolve");
   if (L.angles) {
     launch_k(pdl, k_angles<T>, L.match_grid > 0 ? L.match_grid : 1, 256, 0, s, L.P, L.ctl, (const RepDev*)L.reps,
@@ -2780,16 +2946,15 @@ static void step_impl(const StepLaunch& L, cudaStream_t s, KernelTimer* timer) {
     mark("k_angles");
   }
   const int nbp = (int)((L.cap_particles + kCompactTile - 1) / kCompactTile);
-  const size_t hist_bytes = L.n_counts <= kSmemCounts ? (size_t)L.n_counts * 4 : 0;
   // small systems: 1024 threads per tile (more independent placements per tile); large ones 256
   if (L.cap_particles <= (int64_t)1 << 20)
-    launch_k(pdl, k_compact<T, 1024>, nbp, 1024, hist_bytes, s, L.P, L.ctl, L.reps, (const RepX*)L.repx, L.rep_cons,
-             L.rep_prod, x0, x1, L.id_cur, L.status, prod, L.agg64, L.incl64, L.flags + L.flag_stride, xo, L.id_next,
-             L.counts, L.n_counts, L.history, L.history_len);
+    launch_k(pdl, k_compact<T, 1024>, nbp, 1024, 0, s, L.P, L.ctl, L.reps, (const RepX*)L.repx, L.rep_cons, L.rep_prod,
+             x0, x1, L.id_cur, L.status, prod, (const uint2*)L.events, L.agg64, L.incl64, L.flags + L.flag_stride, xo, L.id_next,
+             L.counts, L.history, L.history_len, (uint32_t)L.cap_particles);
   else
-    launch_k(pdl, k_compact<T, 256>, nbp, 256, hist_bytes, s, L.P, L.ctl, L.reps, (const RepX*)L.repx, L.rep_cons,
-             L.rep_prod, x0, x1, L.id_cur, L.status, prod, L.agg64, L.incl64, L.flags + L.flag_stride, xo, L.id_next,
-             L.counts, L.n_counts, L.history, L.history_len);
+    launch_k(pdl, k_compact<T, 256>, nbp, 256, 0, s, L.P, L.ctl, L.reps, (const RepX*)L.repx, L.rep_cons, L.rep_prod,
+             x0, x1, L.id_cur, L.status, prod, (const uint2*)L.events, L.agg64, L.incl64, L.flags + L.flag_stride, xo, L.id_next,
+             L.counts, L.history, L.history_len, (uint32_t)L.cap_particles);
   mark("k_compact");
 }
 
@@ -2858,10 +3023,11 @@ __global__ void k_set_state(const DevParams* __restrict__ Pp, const RepDev* __re
 // Replica segments and control words of an accepted state (one block; nothing if *err).
 __global__ void k_set_state_finish(const DevParams* __restrict__ Pp, RepDev* __restrict__ reps, DevCtl* __restrict__ ctl,
                                    const uint32_t* __restrict__ cnt, const uint32_t* __restrict__ maxid,
-                                   const uint32_t* __restrict__ next_id_in, const int32_t* __restrict__ err, int64_t n,
+                                   const uint32_t* __restrict__ next_id_in, int32_t* __restrict__ err, int64_t n,
                                    int64_t step) {
   __shared__ unsigned long long sm[32];
   if (*err) return;
+  __syncthreads();
   const DevParams& P = *Pp;
   unsigned long long carry = 0;
   for (int base = 0; base < P.n_replicas; base += blockDim.x) {
@@ -2877,6 +3043,10 @@ __global__ void k_set_state_finish(const DevParams* __restrict__ Pp, RepDev* __r
     carry += tot;
   }
   if (threadIdx.x == 0) {
+    if (ctl->status) {
+      *err = 2;                     // the host resets what an aborted step may have left behind
+      ctl->bar_count = ctl->bar2_count = 0u;
+    }
     ctl->n = (uint32_t)n;
     ctl->step = (uint32_t)step;
     ctl->t = (double)step * P.dt;
@@ -2956,12 +3126,16 @@ __global__ void k_zero_counts(unsigned long long* __restrict__ counts, int n_cou
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_counts; i += gridDim.x * blockDim.x) counts[i] = 0;
 }
 
-// history entry of the current step from the counts (after initialisation or a state upload)
-__global__ void k_history_now(const DevParams* __restrict__ Pp, const DevCtl* __restrict__ ctl,
+// species totals and history entry of the current step from the counts (after initialisation or a state
+// upload)
+__global__ void k_history_now(const DevParams* __restrict__ Pp, DevCtl* __restrict__ ctl,
                               const unsigned long long* __restrict__ counts, long long* __restrict__ history,
                               int history_len) {
   const int ns = Pp->n_species;
-  species_totals(counts, Pp->n_replicas, ns, history + (size_t)(ctl->step % (uint32_t)history_len) * ns);
+  species_totals(counts, Pp->n_replicas, ns, ctl->tot);
+  __syncthreads();
+  for (int k = threadIdx.x; k < ns; k += blockDim.x)
+    history[(size_t)(ctl->step % (uint32_t)history_len) * ns + k] = ctl->tot[k];
 }
 
 void launch_count(const StepLaunch& L, cudaStream_t s) {

@@ -11,13 +11,15 @@
 
 namespace rd {
 
+constexpr int kScanTile = 2048;      // cells per tile of the cell scan
+constexpr int kCompactTile = 2048;   // particles per compaction tile (the look-back buffers are sized for it)
+
 // Device buffers and sizes of one step (pointers are device addresses).
 struct StepLaunch {
   int precision;
   int dim;
   int block;
   int max_grid;
-  int scan_items;
   bool pdl;                    // programmatic dependent launch between the step kernels
   int match_grid;              // blocks of the cooperative matching launch (all resident)
   int fused;                   // 1: the whole step as one cooperative launch (k_step_fused)
@@ -42,8 +44,6 @@ struct StepLaunch {
   uint32_t* id_cur;
   uint32_t* id_next;
   void* x1;
-  void* sx0;                 // cell-ordered start / end positions, interleaved: record k at sx0[2k],
-  void* sx1;                 // sx1[2k] (sx1 = sx0 + one record)
   void* prodpos;
   uint32_t* status;
   int32_t* matched;
@@ -52,7 +52,7 @@ struct StepLaunch {
   uint32_t* slot;
   uint32_t* cell_count;
   uint32_t* cell_start;
-  uint32_t* sidx;
+  float4* rec;                 // cell-ordered records: FP32 start position, particle index (and species)
   uint32_t* decay_list;
   uint32_t* agg32;             // per-tile aggregates / inclusive prefixes of the cell scan
   uint32_t* incl32;
@@ -66,6 +66,7 @@ struct StepLaunch {
   uint32_t* conflict;
   unsigned long long* best_key;
   unsigned long long* best_pid;
+  uint2* events;               // consumed particles of the step: index, products it owns
   unsigned long long* counts;
   long long* history;          // history_len x n_species totals per step (ring), may be null
   int history_len;

@@ -336,16 +336,19 @@ __device__ __noinline__ double lap_p_enc2_warp(double R, double R0, double tau) 
   return p < 0.0 ? 0.0 : (p > 1.0 ? 1.0 : p);
 }
 
-// Upper bound of the 2D p_enc.  u(R) = sqrt(R) g obeys the 1D diffusion equation plus the growth term
-// u / 4R^2, so g_abs is at least the 1D absorbing kernel over sqrt(R R0):
-//   1 - p_enc >= (1 - e^{-(R-1)(R0-1)/tau}) / m,  m = sqrt(2 pi z) e^{-z} I0(z), z = R R0/2tau.
-// Evaluated in FP32 with a margin far above its rounding.
-__device__ __forceinline__ float p_enc2_bound(double R, double R0, double inv_tau) {
-  if (R <= 1.0 || R0 <= 1.0) return 2.0f;
-  const float z = (float)(R * R0 * 0.5 * inv_tau), x = (float)((R - 1.0) * (R0 - 1.0) * inv_tau);
+// FP32 value that the FP64 step's encounter draw must lie below for the pair to need its exact p_enc,
+// from the contact distances d = R - 1 > 0 and d0 = R0 - 1 rounded to FP32 (errors about 1e-6).
+// 3D: the FP32 closed form.  2D: a closed upper bound: u(R) = sqrt(R) g obeys the 1D diffusion equation
+// plus the growth term u / 4R^2, so g_abs is at least the 1D absorbing kernel over sqrt(R R0),
+//   1 - p_enc >= (1 - e^{-d d0/tau}) / m,  m = sqrt(2 pi z) e^{-z} I0(z), z = R R0/2tau.
+// The margin of 1e-4 is far above the rounding of either.
+__device__ __forceinline__ float p_enc_screen(int dim, float d, float d0, float inv_tau) {
+  if (d0 <= 0.0f) return 2.0f;
+  if (dim == 3) return p_enc3_f(d, d0, inv_tau) + 1e-4f;
+  const float z = (1.0f + d) * (1.0f + d0) * 0.5f * inv_tau;
   const float m = z < 40.0f ? sqrtf(6.2831853f * z) * expf(-z) * cyl_bessel_i0f(z)
                             : 1.0f + 0.125f / z + 0.0703125f / (z * z) + 0.0732422f / (z * z * z);
-  return 1.0f + expm1f(-x) / m + 1e-4f;
+  return 1.0f + expm1f(-d * d0 * inv_tau) / m + 1e-4f;
 }
 
 // Eq. (psurv_radII) in 2D.  Warp-collective.
