@@ -434,9 +434,11 @@ static cudaError_t build_tables(rd_handle* h, Alloc alloc) {
       const size_t bytes = (size_t)n0 * m1 * sizeof(float);
       float* t = (float*)alloc(bytes);
       float4* q4 = (float4*)alloc(4 * bytes);
+      float4* q8 = kind == 0 ? (float4*)alloc(8 * bytes) : nullptr;     // rd_pair_probs reads p_reac in pairs of rows
       double* tot = (double*)alloc((size_t)n0 * sizeof(double));
-      if (!t || !q4 || !tot) return cudaErrorMemoryAllocation;
-      launch_build_table(h->L.P, k, kind, t, q4, n0, m1, hstep, h1, tot, fwd, device_sms(), h->stream);
+      if (!t || !q4 || !tot || (kind == 0 && !q8)) return cudaErrorMemoryAllocation;
+      launch_build_table(h->L.P, k, kind, t, q4, q8, n0, m1, hstep, h1, tot, fwd, device_sms(), h->stream);
+      T.q2 = q8;
       T.v = t;
       T.q = q4;
       T.n0 = n0;
@@ -1666,7 +1668,7 @@ extern "C" int rd_step_static(const rd_config* cfg, void* stream, int64_t n, con
   }
   RD_CUDA(cudaMemcpyAsync((void*)L.P, &hp0, sizeof(DevParams), cudaMemcpyHostToDevice, s));
   for (const TableJob& j : jobs)
-    launch_build_table(L.P, j.rule, j.kind, j.t, j.q4, j.n0, j.m1, j.hstep, j.h1, j.tot, nullptr, device_sms(), s);
+    launch_build_table(L.P, j.rule, j.kind, j.t, j.q4, nullptr, j.n0, j.m1, j.hstep, j.h1, j.tot, nullptr, device_sms(), s);
   if (!jobs.empty()) RD_CUDA(cudaMemcpyAsync((void*)L.P, &tmp.hp, sizeof(DevParams), cudaMemcpyHostToDevice, s));
   RD_CUDA(cudaMemcpyAsync(L.reps, &rep, sizeof rep, cudaMemcpyHostToDevice, s));
   RD_CUDA(cudaMemcpyAsync(L.ctl, &ctl, sizeof ctl, cudaMemcpyHostToDevice, s));

@@ -242,6 +242,7 @@ __global__ void __launch_bounds__(128) k_first_passage(const FptArgs A, const do
                                                        double* __restrict__ r_hi, uint32_t* __restrict__ attempts,
                                                        FptItem* __restrict__ queue, uint32_t* __restrict__ qctl,
                                                        uint32_t budget) {
+  pdl_enter();
   const uint32_t lane = threadIdx.x & 31u;
   const double inv_sigma = 1.0 / A.sigma;
   using real = fpt_real<F32>;
@@ -330,6 +331,7 @@ __global__ void __launch_bounds__(128) k_first_passage_warp(const FptArgs A, con
                                                             int next_word, FptItem* __restrict__ queue_out,
                                                             int out_word, uint32_t* __restrict__ qctl,
                                                             uint32_t budget) {
+  pdl_enter();
   const uint32_t lane = threadIdx.x & 31u;
 #pragma unroll 1
   for (;;) {
@@ -456,6 +458,7 @@ __global__ void __launch_bounds__(kFptBlockThreads) k_first_passage_block(
   __shared__ uint32_t s_item, s_win;
   __shared__ double s_rm;
   __shared__ int s_dec;
+  pdl_enter();
   const uint32_t tid = threadIdx.x;
 #pragma unroll 1
   for (;;) {
@@ -503,6 +506,7 @@ __global__ void __launch_bounds__(kFptGridThreads) k_first_passage_grid(
     double* __restrict__ r_hi, uint32_t* __restrict__ attempts, const FptItem* __restrict__ queue,
     FptSearch* __restrict__ search, FptItem* __restrict__ queue_next, uint32_t* __restrict__ qctl, int words) {
   __shared__ uint32_t s_chunk, s_stop, s_last;
+  pdl_enter();
   const uint32_t tid = threadIdx.x, nt = blockDim.x;
   const uint32_t count = qctl[words + kFptGridIn];
   // the grid works in groups of blocks (block index mod groups); group g takes items g, g + groups, ...
@@ -585,12 +589,13 @@ static void launch_fpt(const FptArgs& A, const double* r0, const double* r, cons
   // more at a later level; a round with nothing queued ends at once
   for (int round = 0; round < A.levels; ++round) {
     const int w = kFptRound0 + round * kFptRoundWords;
-    k_first_passage_warp<F32><<<gw, 128, 0, s>>>(A, stream, bin, r_lo, r_hi, attempts, warp_q[round & 1], w + kFptWarpIn,
-                                            w + kFptWarpNext, block_q, w + kFptBlockIn, qctl, kFptWarpBudget);
-    k_first_passage_block<F32><<<gb, kFptBlockThreads, 0, s>>>(A, stream, bin, r_lo, r_hi, attempts, block_q, grid_q,
-                                                          search, qctl, w, kFptBlockBudget);
-    k_first_passage_grid<F32><<<gb, kFptGridThreads, 0, s>>>(A, stream, bin, r_lo, r_hi, attempts, grid_q, search,
-                                                        warp_q[(round + 1) & 1], qctl, w);
+    launch_k(true, k_first_passage_warp<F32>, (int)gw, 128, 0, s, A, stream, bin, r_lo, r_hi, attempts,
+             (const FptItem*)warp_q[round & 1], w + kFptWarpIn, w + kFptWarpNext, block_q, w + kFptBlockIn, qctl,
+             kFptWarpBudget);
+    launch_k(true, k_first_passage_block<F32>, (int)gb, kFptBlockThreads, 0, s, A, stream, bin, r_lo, r_hi, attempts,
+             (const FptItem*)block_q, grid_q, search, qctl, w, kFptBlockBudget);
+    launch_k(true, k_first_passage_grid<F32>, (int)gb, kFptGridThreads, 0, s, A, stream, bin, r_lo, r_hi, attempts,
+             (const FptItem*)grid_q, search, warp_q[(round + 1) & 1], qctl, w);
   }
 }
 

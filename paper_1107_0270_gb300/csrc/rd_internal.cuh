@@ -19,6 +19,16 @@ constexpr uint32_t kRecIndex = 0x0FFFFFFFu;      // particle index in a packed c
 constexpr uint32_t kOneParticle = 0xFFFFFFFFu;   // id_b of one-particle random streams
 constexpr uint32_t kMaxEvents = 4096;            // consumed particles of a step that the event list holds
 
+#ifdef __CUDACC__
+// Programmatic dependent launch: a kernel waits for the whole previous kernel (completion and memory
+// visibility) before it touches memory, then lets the next kernel's blocks be scheduled while its own
+// blocks run.  Both are no-ops for a launch without a programmatic dependency.
+__device__ __forceinline__ void pdl_enter() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+
 // Random-stream tags (counter word 3, low byte; replica index in the upper 24 bits).
 enum Tag : uint32_t {
   TAG_INIT0 = 1, TAG_INIT1 = 2, TAG_UNI = 3, TAG_DISP0 = 4, TAG_DISP1 = 5, TAG_ENC = 6,
@@ -49,6 +59,8 @@ struct Series2D;
 struct Tab2 {
   const float* v;             // n0 x n1 values on the grid (x0, x1) = (h (i-1), h1 (j-1))
   const float4* q;            // q[i n1 + j] = v[i n1 + j-1 .. j+2]: one aligned load per stencil row
+  const float4* q2;           // q2[2 (i n1 + j)] = q[i n1 + j], q[(i+1) n1 + j]: two stencil rows in one 32-byte
+                              // sector (null: not built)
   int32_t n0, n1;
   float inv_h, h;             // first axis
   float inv_h1, h1;           // second axis
@@ -310,6 +322,39 @@ __device__ __forceinline__ double norm2_rn(double a, double b, double c, int dim
   return s;
 }
 
+// Double <-> float conversions on the integer pipe (the hardware conversions run on the FP64 pipe, two
+// lanes per SM and cycle).  narrow_rn: the double rounded to nearest even, by the instruction outside
+// FP32's normal range; widen: a float that is not negative, exactly (NaN stays NaN).
+__device__ __forceinline__ float narrow_rn(double a) {
+  const uint32_t hi = (uint32_t)__double2hiint(a), lo = (uint32_t)__double2loint(a);
+  if (hi - 0x38100000u >= 0x0FD00000u) {      // outside [2^-126, 2^127)
+    float f;
+    asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(f) : "d"(a));
+    return f;
+  }
+  const uint32_t m = __funnelshift_l(lo, hi - 0x38000000u, 3);
+  return __uint_as_float(m + (((lo & 0x1FFFFFFFu) + 0x0FFFFFFFu + (m & 1u)) >> 29));
+}
+__device__ __forceinline__ double widen(float a) {
+  const bool small = a < 0x1p-126f;            // subnormal or zero: scaled exactly into the normal range
+  const uint32_t u = __float_as_uint(small ? a * 0x1p64f : a);
+  uint32_t hi = (u >> 3) + (small ? 0x38000000u - (64u << 20) : 0x38000000u);
+  if (u == 0u) hi = 0u;
+  if (u >= 0x7F800000u) hi = u == 0x7F800000u ? 0x7FF00000u : 0x7FF80000u;
+  return __hiloint2double((int)hi, (int)(u << 29));
+}
+// 32 bytes (32-byte aligned) in one load.
+struct f8 {
+  float4 a, b;
+};
+__device__ __forceinline__ f8 ldg_f8(const float4* p) {
+  f8 v;
+  asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=f"(v.a.x), "=f"(v.a.y), "=f"(v.a.z), "=f"(v.a.w), "=f"(v.b.x), "=f"(v.b.y), "=f"(v.b.z), "=f"(v.b.w)
+      : "l"(p));
+  return v;
+}
+
 __device__ __forceinline__ uint32_t w_bits(double w) { return (uint32_t)__double_as_longlong(w); }
 __device__ __forceinline__ uint32_t w_bits(float w) { return __float_as_uint(w); }
 __device__ __forceinline__ double w_from_bits_d(uint32_t b) { return __longlong_as_double((long long)b); }
@@ -537,7 +582,30 @@ __device__ __forceinline__ float tab_eval(const Tab2& T, float d0, float d) {
   return acc;
 }
 
+// tab_eval on the paired rows: the same values and arithmetic from two 32-byte loads instead of four
+// 16-byte ones.  (A batch of unrelated pairs is bound by the L1's one line per lane and load.)
+__device__ __forceinline__ float tab_eval2(const Tab2& T, float d0, float d) {
+  float x = d0 * T.inv_h + 1.0f, y = d * T.inv_h1 + 1.0f;
+  x = fminf(fmaxf(x, 1.0f), (float)(T.n0 - 3) - 1e-3f);
+  y = fminf(fmaxf(y, 1.0f), (float)(T.n1 - 3) - 1e-3f);
+  const int i = (int)x, j = (int)y;
+  float wx[4], wy[4];
+  cr_w(x - i, wx);
+  cr_w(y - j, wy);
+  const float4* p = T.q2 + 2 * ((size_t)(i - 1) * T.n1 + j);
+  const f8 lo = ldg_f8(p), hi = ldg_f8(p + 4 * (size_t)T.n1);
+  const float4 v[4] = {lo.a, lo.b, hi.a, hi.b};
+  float acc = 0.0f;
+#pragma unroll
+  for (int a = 0; a < 4; ++a) acc += wx[a] * (wy[0] * v[a].x + wy[1] * v[a].y + wy[2] * v[a].z + wy[3] * v[a].w);
+  return acc;
+}
+
 // table p_reac (clamped to [0,1])
+__device__ __forceinline__ float p_reac_tab2(const PairDev& pr, float d, float d0) {
+  const float p = tab_eval2(pr.tab_preac, fmaxf(d0, 0.0f), fmaxf(d, 0.0f));
+  return fminf(fmaxf(p, 0.0f), 1.0f);
+}
 __device__ __forceinline__ float p_reac_tab(const PairDev& pr, float d, float d0) {
   const float p = tab_eval(pr.tab_preac, fmaxf(d0, 0.0f), fmaxf(d, 0.0f));
   return fminf(fmaxf(p, 0.0f), 1.0f);

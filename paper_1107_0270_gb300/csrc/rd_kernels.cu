@@ -14,15 +14,6 @@
 
 namespace rd {
 
-// Programmatic dependent launch: a step kernel waits for the whole previous kernel (completion and
-// memory visibility) before it touches memory, then lets the next kernel's blocks be scheduled while
-// its own blocks run.  Both are no-ops for a launch without a programmatic dependency.
-__device__ __forceinline__ void pdl_enter() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
-
 // Acquire load / release store of a 32-bit flag at GPU scope (the look-back's and the grid
 // barrier's publication protocol: data written before a release store is visible to whoever
 // acquires the flag value it stored).
@@ -2044,8 +2035,10 @@ __device__ __forceinline__ void ph_angles(const DevParams* Pp, DevCtl* ctl,
       ang_job_place<T>(j, reps[j.r], dim, dir, x1, prodpos);
     }
   }
+  // (consecutive blocks start on different warps: neighbouring blocks share an SM, and an SM quadrant
+  // issues one FP64 instruction in 64 cycles)
   const uint32_t wpb = blockDim.x >> 5, wid = threadIdx.x >> 5;
-  for (uint32_t q = wid * nblk + bid; q < nj; q += nblk * wpb) {
+  for (uint32_t q = ((wid + wpb - bid % wpb) % wpb) * nblk + bid; q < nj; q += nblk * wpb) {
     const AngJob& j = jobs[q];
     if (sizeof(T) == 4 && P.pairs[j.kind >> 8].tab_ang.v) continue;
     const double v = lap_ang_sample_warp(dim, j.U_ang, j.Rn, j.R0, j.tau, s_dn[wid]);
@@ -2449,10 +2442,10 @@ __device__ __forceinline__ void pair_probs_one(const DevParams& P, const PairDev
                                                double& prc, bool want_enc, bool want_reac) {
   // mixed: the separations rounded once to FP32 and scaled there (FP64 arithmetic runs at 1/64 of
   // the FP32 rate on this part)
-  const float d0 = fmaf((float)a, pr.inv_sigma_f, -1.0f), d = fmaf((float)b, pr.inv_sigma_f, -1.0f);
+  const float d0 = fmaf(narrow_rn(a), pr.inv_sigma_f, -1.0f), d = fmaf(narrow_rn(b), pr.inv_sigma_f, -1.0f);
   if (want_enc) {
     if (kMixed3D) {
-      pe = (double)p_enc3_f(d, d0, pr.inv_tau_f);
+      pe = widen(p_enc3_f(d, d0, pr.inv_tau_f));
     } else if (P.precision == RD_MIXED) {
       float pf;
       if (P.dim == 3) {
@@ -2472,7 +2465,7 @@ __device__ __forceinline__ void pair_probs_one(const DevParams& P, const PairDev
     double v = pr.bc == RD_BC_ABS ? 1.0 : 0.0;
     if (pr.bc == RD_BC_RAD) {
       if (kMixed3D)
-        v = (double)p_reac_tab(pr, d, d0);
+        v = widen(p_reac_tab2(pr, d, d0));
       else
         v = P.precision == RD_MIXED ? (double)p_reac_tab(pr, d, d0) : p_reac_dim(P, pr, b / pr.sigma, a / pr.sigma);
     }
@@ -2659,13 +2652,18 @@ __global__ void k_table_ghost_row(float* __restrict__ T, int n1) {
 }
 
 // quad layout of a finished table: q[i n1 + j] = (v[i n1 + j-1], .., v[i n1 + j+2]), zero off the ends
-__global__ void k_table_quads(const float* __restrict__ T, int n0, int n1, float4* __restrict__ Q) {
+__global__ void k_table_quads(const float* __restrict__ T, int n0, int n1, float4* __restrict__ Q,
+                              float4* __restrict__ Q2) {
   const int64_t total = (int64_t)n0 * n1;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total; k += (int64_t)gridDim.x * blockDim.x) {
     const int j = (int)(k % n1);
     float4 q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (j >= 1 && j + 2 < n1) q = make_float4(T[k - 1], T[k], T[k + 1], T[k + 2]);
     Q[k] = q;
+    if (Q2) {
+      Q2[2 * k] = q;
+      if (k >= n1) Q2[2 * (k - n1) + 1] = q;
+    }
   }
 }
 
@@ -2690,7 +2688,7 @@ __global__ void k_build_inverse2(Tab2 fwd, float* __restrict__ out, int n0, int 
   }
 }
 
-void launch_build_table(const DevParams* P, int rule, int kind, float* out, float4* quad, int n0, int n1, double h,
+void launch_build_table(const DevParams* P, int rule, int kind, float* out, float4* quad, float4* quad2, int n0, int n1, double h,
                         double h1, double* tot, const Tab2* fwd, int device_sms, cudaStream_t s) {
   if (kind == 2) k_tail_totals<<<(n0 + 63) / 64, 64, 0, s>>>(P, rule, n0, h, tot);
   const int64_t total = (int64_t)n0 * n1;
@@ -2701,7 +2699,7 @@ void launch_build_table(const DevParams* P, int rule, int kind, float* out, floa
     k_build_table<<<G, 128, 0, s>>>(P, rule, kind, out, n0, n1, h, h1, tot);
   k_table_ghosts<<<(n0 + 255) / 256, 256, 0, s>>>(out, n0, n1);
   k_table_ghost_row<<<(n1 + 255) / 256, 256, 0, s>>>(out, n1);
-  k_table_quads<<<G, 128, 0, s>>>(out, n0, n1, quad);
+  k_table_quads<<<G, 128, 0, s>>>(out, n0, n1, quad, quad2);
 }
 
 // ================================================================================================
@@ -2838,23 +2836,6 @@ static inline int grid_for(int64_t n, int block, int max_grid) {
   if (g < 1) g = 1;
   if (g > max_grid) g = max_grid;
   return (int)g;
-}
-
-// Kernel launch with the programmatic-stream-serialization attribute (see pdl_enter).
-template <typename... KArgs, typename... Args>
-static void launch_k(bool pdl, void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s,
-                     Args&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
 // Cooperative launch (all blocks resident at once, as the grid barrier requires; a grid larger

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "rd_internal.cuh"
@@ -95,6 +96,23 @@ struct KernelTimer {
   }
 };
 
+// Kernel launch with the programmatic-stream-serialization attribute (see pdl_enter).
+template <typename... KArgs, typename... Args>
+static inline void launch_k(bool pdl, void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s,
+                     Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
 // blocks of the cooperative matching launch that fit on the device at once (>= 1)
 int match_grid_size(int device_sms);
 // blocks of the fused step launch for L's precision, sweep split and reach that fit on the device
@@ -123,7 +141,8 @@ void launch_count(const StepLaunch& L, cudaStream_t s);
 void launch_pair_probs(const DevParams* P, int rule, const double* r0, const double* r, int64_t n, double* pe,
                        double* pr, int max_grid, bool mixed3d, cudaStream_t s);
 // kind 3 with fwd != nullptr: the 2D inverse table from the forward -ln(tail) table fwd
-void launch_build_table(const DevParams* P, int rule, int kind, float* out, float4* quad, int n0, int n1, double h,
+// (quad2: the paired rows of Tab2::q2, or null)
+void launch_build_table(const DevParams* P, int rule, int kind, float* out, float4* quad, float4* quad2, int n0, int n1, double h,
                         double h1, double* tot, const Tab2* fwd, int device_sms, cudaStream_t s);
 // warp: one warp per draw (FP64 in 2D), else one thread
 void launch_resample(const DevParams* P, int rule, const double* r0, const double* u, int64_t n, double* out,
@@ -151,9 +170,13 @@ struct FptArgs {
   const void* ser;             // 2D small-time series coefficients of the rule
   FptLevel lv[kFptMaxLevels];
 };
-constexpr uint32_t kFptBudget = 256;        // draws per pair in the lane-per-pair phase
-constexpr uint32_t kFptWarpBudget = 4352;   // draws per pair before the block-per-pair phase
-constexpr uint32_t kFptBlockBudget = 32768; // draws per pair before the grid phase
+// Where a pair moves on.  A lane draws one attempt at a time, about 3000 cycles each once the other lanes
+// have finished, so a large first budget is a long tail with few lanes busy; a small one sends pairs to a
+// warp that would have finished soon.  2^20 pairs, 10 levels, FP32 / FP64: 256, 4352, 32768 2.27 / 41 ms;
+// 64, 1024, 16384 1.38 / 29; 48, 512, 8192 1.30 / 27.8; 24, 384, 4096 1.38 / 31.
+constexpr uint32_t kFptBudget = 48;         // draws per pair in the lane-per-pair phase
+constexpr uint32_t kFptWarpBudget = 512;    // further draws before the block-per-pair phase
+constexpr uint32_t kFptBlockBudget = 8192;  // further draws before the grid phase
 constexpr int kFptBlockThreads = 512;       // threads per pair in the block-per-pair phase
 constexpr int kFptGridThreads = 256;        // threads per block (and attempts per chunk) of the grid phase
 constexpr uint32_t kFptGridGroups = 4;      // block groups of the grid phase, each searching its own pairs

@@ -418,7 +418,8 @@ __device__ __noinline__ double lap_resample2_warp(double U, double R0, double ta
     else
       hi = V;
     double Vn = tail > 0.0 && den > 0.0 ? V + y * tail / den : -1.0;
-    const bool inside = Vn > lo && Vn < hi;
+    // (a step that rounds to the bracket's end has converged)
+    const bool inside = Vn >= lo && Vn <= hi;
     if (!inside) Vn = 0.5 * (lo + hi);
     const double step = fabs(Vn - V);
     V = Vn;
