@@ -449,13 +449,16 @@ constexpr double kFilter = 1e-4;
 // With w = R0-1, z = (V+w)/2s, z0 = w/2s, the normalised tail beyond R = 1 + V is
 //   T(V) = exp(z0^2 - z^2) [erfcx(z) + V erfcx(s+z)] / erfcx(z0),
 //   d ln T / dV = -(1+V) [q(s+z) + sqrt(pi) z erfcx(s+z)] / (s sqrt(pi) [erfcx(z) + V erfcx(s+z)]).
+// d2: the second derivative over the first (the tail's density rho obeys rho'/rho = 1/(1+V) - z/s + q/B
+// with B the bracket of d ln T / dV, since dB/dV = q).
 __device__ __forceinline__ void lnT3(double V, double w, double s, double inv_4tau, double ln_ex0,
-                                     double& f, double& df) {
+                                     double& f, double& df, double& d2) {
   const double z = (V + w) / (2.0 * s);
   const double ez = erfcx(z), y = s + z, ey = erfcx(y);
-  const double body = ez + V * ey;
+  const double body = ez + V * ey, q = q_ierfc(y, ey), B = q + kSqrtPi * z * ey;
   f = -V * (2.0 * w + V) * inv_4tau + log(body) - ln_ex0;
-  df = -(1.0 + V) * (q_ierfc(y, ey) + kSqrtPi * z * ey) / (s * kSqrtPi * body);
+  df = -(1.0 + V) * B / (s * kSqrtPi * body);
+  d2 = 1.0 / (1.0 + V) - z / s + q / B - df;
 }
 
 // FP32 evaluation of ln T and its derivative (the FP64 solve's seed; the mixed step's Newton step).
@@ -492,10 +495,11 @@ __device__ __forceinline__ float resample3_seed(double U, double R0, double s) {
   return Vf >= 0.0f && isfinite(Vf) ? Vf : 0.0f;
 }
 
-// Solves ln T(V) = ln U.  A few FP32 Newton steps give a seed good to ~1e-5; FP64 Newton steps,
-// each kept inside the bracket known so far (bisection / expansion otherwise), finish the solve.
-// Once an FP64 Newton step is below 1e-10 of the length scale max(V, s), quadratic convergence
-// makes the new iterate accurate to rounding.
+// Solves ln T(V) = ln U.  A few FP32 Newton steps give a seed good to ~1e-5; FP64 Halley steps (third
+// order: the second derivative costs two divisions where an evaluation of ln T costs two erfcx and a
+// logarithm), each kept inside the bracket known so far (bisection / expansion otherwise), finish the
+// solve.  Once a step is below 1e-5 of the length scale max(V, s), the new iterate is accurate to
+// rounding: mostly one evaluation, where Newton steps took three.
 __device__ __forceinline__ double resample3(double U, double R0, double s) {
   if (R0 < 1.0) R0 = 1.0;
   const double w = R0 - 1.0;
@@ -504,21 +508,23 @@ __device__ __forceinline__ double resample3(double U, double R0, double s) {
   const float Vf = resample3_seed(U, R0, s);
   const double ln_ex0 = log(erfcx(w / (2.0 * s)));
   double lo = 0.0, hi = -1.0;          // hi < 0: no upper bound yet
-  double V = (double)Vf, f = 0.0, df;
+  double V = (double)Vf, f = 0.0, df, d2;
   for (int it = 0; it < 200; ++it) {
-    lnT3(V, w, s, inv_4tau, ln_ex0, f, df);
+    lnT3(V, w, s, inv_4tau, ln_ex0, f, df, d2);
     const double g = f - lnU;
     if (g == 0.0) break;
     if (g > 0.0)
       lo = V;
     else
       hi = V;
-    double Vn = V - g / df;
+    const double nt = g / df;
+    const double hl = 1.0 - 0.5 * nt * d2;
+    double Vn = V - (hl > 0.5 ? nt / hl : nt);
     const bool inside = Vn >= lo && (hi < 0.0 || Vn <= hi);
     if (!inside) Vn = hi < 0.0 ? lo + fmax(lo, s) : 0.5 * (lo + hi);
     const double step = fabs(Vn - V);
     V = Vn;
-    if (inside && step <= 1e-10 * fmax(V, s)) break;
+    if (inside && step <= 3e-6 * fmin(V, s) + 1e-10 * s) break;
     if (hi >= 0.0 && hi - lo <= 4e-16 * fmax(hi, s)) break;
   }
   return 1.0 + V;

@@ -490,7 +490,7 @@ __device__ __forceinline__ void ph_sweep(const DevParams* Pp, DevCtl* ctl,
                                          const int64_t total_cells, FiredPair* fired,
                                          uint32_t* fstate, uint32_t* deg,
                                          int32_t* matched, const uint32_t cap_pairs,
-                                         const uint32_t split, uint2 (*ranges)[256],
+                                         const uint32_t split, const uint32_t per_block, uint2 (*ranges)[256],
                                          const uint32_t bid, const uint32_t nblk) {
   // per-warp queue of (particle, candidate) pairs that passed the cut-off test
   __shared__ uint2 s_queue[8][64];
@@ -662,10 +662,10 @@ __device__ __forceinline__ void ph_sweep(const DevParams* Pp, DevCtl* ctl,
   // split = 1: one thread walks all rows of a particle; split = number of rows: one thread per
   // (particle, row), more independent chains for small systems (the host keeps nb * split < 2^32)
   const uint32_t work = kSplit ? nb * split : nb;
-  const uint32_t stride = nblk * blockDim.x;
+  const uint32_t stride = nblk * per_block;
   const uint32_t n_iter = (work + stride - 1) / stride;
   for (uint32_t it = 0; it < n_iter; ++it) {
-    const uint32_t t = it * stride + bid * blockDim.x + threadIdx.x;
+    const uint32_t t = threadIdx.x < per_block ? it * stride + bid * per_block + threadIdx.x : work;
     int nr = 0;
     uint32_t k = 0, me = 0, mask = 0;
     float ax = 0.0f, ay = 0.0f, az = 0.0f, Lf = 0.0f, hLf = 0.0f, cut = 0.0f;
@@ -784,11 +784,11 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 5) k_sweep(const Dev
                                                   const int64_t total_cells, FiredPair* __restrict__ fired,
                                                   uint32_t* __restrict__ fstate, uint32_t* __restrict__ deg,
                                                   int32_t* __restrict__ matched, const uint32_t cap_pairs,
-                                                  const uint32_t split) {
+                                                  const uint32_t split, const uint32_t per_block) {
   pdl_enter();
   __shared__ uint2 ranges[kSweepRanges][256];
   ph_sweep<T, kSplit, kReach>(Pp, ctl, reps, x0, x1, id, rec, cell_start, total_cells, fired, fstate, deg, matched,
-                              cap_pairs, split, ranges, blockIdx.x, gridDim.x);
+                              cap_pairs, split, per_block, ranges, blockIdx.x, gridDim.x);
 }
 
 // ================================================================================================
@@ -2752,7 +2752,7 @@ __global__ void __launch_bounds__(256, 2) k_step_fused(const StepLaunch L, const
     if (!grid_barrier(ctl, false)) return;
     phase_stamp(ctl, 3);
     ph_sweep<T, kSplit, kReach>(L.P, ctl, L.reps, x0s, x1, id0, L.rec, L.cell_start, L.total_cells, L.fired, L.fstate,
-                                L.deg, L.matched, (uint32_t)L.cap_pairs, split, (uint2(*)[256])dsm, blockIdx.x,
+                                L.deg, L.matched, (uint32_t)L.cap_pairs, split, blockDim.x, (uint2(*)[256])dsm, blockIdx.x,
                                 gridDim.x);
     if (!grid_barrier(ctl, false)) return;
     phase_stamp(ctl, 4);
@@ -2909,10 +2909,12 @@ static void step_impl(const StepLaunch& L, cudaStream_t s, KernelTimer* timer) {
   // FP64 in 2D: one-warp blocks, so that the warp-wide p_enc evaluations (the FP64 pipe of an SM is
   // what they wait for) spread over the SMs
   const int Bs = sizeof(T) == 8 && L.dim == 2 ? 32 : 256;
-  const int Gs = grid_for(L.cap_particles * (int64_t)split, Bs, L.max_grid);
+  // ... and, while there are blocks to spare, a quarter of a warp's particles in each
+  const int per_block = Bs == 32 && L.cap_particles * (int64_t)split <= 8 * (int64_t)L.max_grid ? 8 : Bs;
+  const int Gs = grid_for(L.cap_particles * (int64_t)split, per_block, L.max_grid);
   auto sweep = [&](auto kernel) {
     launch_k(pdl, kernel, Gs, Bs, 0, s, L.P, L.ctl, L.reps, x0s, x1, L.id_cur, L.rec, L.cell_start, L.total_cells,
-             L.fired, L.fstate, L.deg, L.matched, (uint32_t)L.cap_pairs, split);
+             L.fired, L.fstate, L.deg, L.matched, (uint32_t)L.cap_pairs, split, (uint32_t)per_block);
   };
   if (L.reach == 2)
     split > 1 ? sweep(k_sweep<T, true, 2>) : sweep(k_sweep<T, false, 2>);

@@ -114,13 +114,16 @@ RD_HD void k01_scaled(cplx x, cplx& k0, cplx& k1) {
   int n = 12 + (int)(280.0 / key);
   if (n > kLapMiller) n = kLapMiller;
   cplx up = cx(0.0, 0.0), u = cx(1e-150, 0.0), sum = u;
+  double n1 = n + 1.0;
+  cplx b = cx(2.0 * (n + x.re), 2.0 * x.im);
 #pragma unroll 1
   for (; n >= 1; --n) {
-    const cplx b = cx(2.0 * (n + x.re), 2.0 * x.im);
-    const cplx v = RD_LAP.r[n] * (b * u - (n + 1.0) * up);
+    const cplx v = RD_LAP.r[n] * (b * u - n1 * up);
     up = u;
     u = v;
     sum = sum + v;
+    b.re -= 2.0;
+    n1 -= 1.0;
   }
   // sqrt(pi / 2x): principal root (Re x > 0)
   const cplx q = (0.5 * kPi) * ix;
@@ -176,6 +179,7 @@ RD_HD LapNode lap_node(double u, double tau, int lane) {
 // The sequences K_n, K_{n+1} (scaled) of one lane's node at the arguments w, R w, R0 w; the weight
 // is folded into the R0 sequence.  step() returns the node's share of D_n and moves on to n + 1.
 struct LapAng {
+  cplx am;                      // K_{n-1} at w (n = 0: its continuation)
   cplx a, a1, b, b1, q, q1;     // K_n, K_{n+1} at w, R w, R0 w
   cplx iw, cw, cr, cq;          // 1/w; (2n+1)/z (3D) or 2n/z (2D) of K_{n+1}'s recurrence, per argument
   cplx dw, dr, dq;              // 2/z
@@ -185,28 +189,32 @@ struct LapAng {
     const cplx ir = (1.0 / R) * iw, iq = (1.0 / R0) * iw;
     if (dim == 3) {
       a = iw; b = ir; q = iq;                                         // e^z k_0 = 1/z
+      am = cx(0.0, 0.0);
       a1 = iw * (cx(1.0, 0.0) + iw); b1 = ir * (cx(1.0, 0.0) + ir); q1 = iq * (cx(1.0, 0.0) + iq);
       cw = iw; cr = ir; cq = iq;
     } else {
       k01_scaled(w, a, a1);
       k01_scaled(wr, b, b1);
       k01_scaled(wq, q, q1);
+      am = a1;
       cw = cr = cq = cx(0.0, 0.0);
     }
     q = q * k.wt;
     q1 = q1 * k.wt;
     dw = 2.0 * iw; dr = 2.0 * ir; dq = 2.0 * iq;
   }
-  RD_HD double step(int n) {
-    // -K_n' = K_{n+1} - (n/z) K_n in both dimensions
-    const cplx kd = a1 - (double)n * (iw * a);
+  // dn = n.  The derivative as the recurrence gives it, -(2n+1) k_n' = n k_{n-1} + (n+1) k_{n+1} (3D),
+  // -2 K_n' = K_{n-1} + K_{n+1} (2D): the share comes out divided by 2n + 1 (3D) or by 2.
+  RD_HD double step(bool d3, double dn) {
+    const cplx kd = d3 ? dn * am + (dn + 1.0) * a1 : am + a1;
     const double c = re_quot(b * q, a * kd);
     cw = cw + dw; cr = cr + dr; cq = cq + dq;
-    cplx t = a + cw * a1; a = a1; a1 = t;
+    am = a;
+    cplx t = am + cw * a1; a = a1; a1 = t;
     t = b + cr * b1; b = b1; b1 = t;
     t = q + cq * q1; q = q1; q1 = t;
     if (fabs(a.re) + fabs(a.im) > 1e60) {      // all three scaled alike: the quotient does not change
-      a = 1e-60 * a; a1 = 1e-60 * a1; b = 1e-60 * b; b1 = 1e-60 * b1; q = 1e-60 * q; q1 = 1e-60 * q1;
+      am = 1e-60 * am; a = 1e-60 * a; a1 = 1e-60 * a1; b = 1e-60 * b; b1 = 1e-60 * b1; q = 1e-60 * q; q1 = 1e-60 * q1;
     }
     return c;
   }
@@ -223,21 +231,25 @@ RD_HD int lap_ang_terms(double kappa, int n_law) {
 // entries).  Returns the last order worth summing.  Warp-collective.
 __device__ __forceinline__ int lap_ang_coeffs_warp(int dim, double R, double R0, double tau, int N, double* Dn) {
   const int lane = threadIdx.x & 31;
+  const bool d3 = dim == 3;
   const LapNode k = lap_node(fmax(R + R0 - 2.0, 0.0), tau, lane);
   LapAng A;
   A.start(dim, k, R, R0);
-  double inv = 0.0;
+  double dn = 0.0, c0 = 0.0;
   int last = 0, small = 0;
 #pragma unroll 1
   for (int n = 0; n <= N; ++n) {
-    double c = warp_sum(A.step(n));
-    if (n == 0) inv = 1.0 / c;
-    c *= inv;
+    const double c = warp_sum(A.step(d3, dn));
+    dn += 1.0;
+    if (n == 0) c0 = c;
     if (lane == 0) Dn[n] = c;
     last = n;
-    small = fabs(c) < 1e-18 ? small + 1 : 0;
+    small = fabs(c) < 1e-20 * fabs(c0) ? small + 1 : 0;
     if (small == 2) break;
   }
+  __syncwarp();
+  const double inv = 1.0 / c0;
+  for (int n = lane; n <= last; n += 32) Dn[n] *= d3 ? (2 * n + 1) * inv : inv;
   __syncwarp();
   return last;
 }
@@ -276,11 +288,45 @@ __device__ __forceinline__ void lap_ang_cdf(int dim, const double* Dn, int N, do
   f = (1.0 + 2.0 * den) * (1.0 / kPi);
 }
 
+// The same in FP32 from the same coefficients (the starting point of the FP64 solution).
+__device__ __forceinline__ void lap_ang_cdf_f(bool d3, const double* Dn, int N, float v, float& F, float& f) {
+  float acc = 0.0f, den = 0.0f;
+  if (d3) {
+    float pm1 = 1.0f, p = v;
+#pragma unroll 1
+    for (int n = 1; n <= N; ++n) {
+      const float d = (float)Dn[n];
+      const float pp1 = (float)c_lap.leg_a[n] * v * p - (float)c_lap.leg_b[n] * pm1;
+      acc += d * (pp1 - pm1);
+      den += (2.0f * n + 1.0f) * d * p;
+      pm1 = p;
+      p = pp1;
+    }
+    F = 0.5f * (1.0f + v) + 0.5f * acc;
+    f = 0.5f * (1.0f + den);
+    return;
+  }
+  float s1, c1;
+  sincosf(v, &s1, &c1);
+  float sn = s1, cn = c1;
+#pragma unroll 1
+  for (int n = 1; n <= N; ++n) {
+    const float d = (float)Dn[n];
+    acc += d * (sn * (float)c_lap.ik[n]);
+    den += d * cn;
+    const float t = sn * c1 + cn * s1;
+    cn = cn * c1 - sn * s1;
+    sn = t;
+  }
+  F = (v + 2.0f * acc) * (float)(1.0 / kPi);
+  f = (1.0f + 2.0f * den) * (float)(1.0 / kPi);
+}
+
 // Angle of the new separation to the start separation at CDF value U (3D its cosine in [-1, 1], 2D the
 // angle in [0, pi]) from the full propagator.  NaN if the law needs more than kAngNMax - 1 partial
 // waves.  Warp-collective, identical arguments in every lane; Dn: kAngNMax doubles of shared memory.
-// Two rounds of 32 trial points narrow the bracket to 1/1089 of the range, Newton steps inside it
-// finish (the CDF is monotonic).
+// Three rounds of 32 trial points in FP32 come within 1e-4 of the range, Newton steps in FP64 inside a
+// bracket finish (the CDF is monotonic); an FP64 evaluation costs a warp about 8000 cycles.
 __device__ __noinline__ double lap_ang_sample_warp(int dim, double U, double R, double R0, double tau, double* Dn) {
   const double kappa = R * R0 / (2.0 * tau);
   const int n_law = ang_terms(kappa);
@@ -288,19 +334,24 @@ __device__ __noinline__ double lap_ang_sample_warp(int dim, double U, double R, 
   __syncwarp();                                   // the previous pair's readers are done with Dn
   const int N = lap_ang_coeffs_warp(dim, R, R0, tau, lap_ang_terms(kappa, n_law), Dn);
   const int lane = threadIdx.x & 31;
-  double lo = dim == 3 ? -1.0 : 0.0, hi = dim == 3 ? 1.0 : kPi, F, f;
+  const float Uf = (float)U;
+  float lof = dim == 3 ? -1.0f : 0.0f, hif = dim == 3 ? 1.0f : (float)kPi, Ff, ff;
 #pragma unroll 1
-  for (int round = 0; round < 2; ++round) {
-    const double st = (hi - lo) * (1.0 / 33.0);
-    lap_ang_cdf(dim, Dn, N, lo + (lane + 1) * st, F, f);
-    const int below = __popc(__ballot_sync(0xFFFFFFFFu, F < U));
-    const double nlo = lo + below * st;
-    hi = below < 32 ? lo + (below + 1) * st : hi;
-    lo = nlo;
+  for (int round = 0; round < 3; ++round) {
+    const float st = (hif - lof) * (1.0f / 33.0f);
+    lap_ang_cdf_f(dim == 3, Dn, N, lof + (lane + 1) * st, Ff, ff);
+    const int below = __popc(__ballot_sync(0xFFFFFFFFu, Ff < Uf));
+    const float nlo = lof + below * st;
+    hif = below < 32 ? lof + (below + 1) * st : hif;
+    lof = nlo;
   }
-  double v = 0.5 * (lo + hi);
+  float vf = 0.5f * (lof + hif);
+  lap_ang_cdf_f(dim == 3, Dn, N, vf, Ff, ff);
+  if (ff > 0.0f) vf = fminf(fmaxf(vf - (Ff - Uf) / ff, lof), hif);
+  double lo = dim == 3 ? -1.0 : 0.0, hi = dim == 3 ? 1.0 : kPi, F, f;
+  double v = fmin(fmax((double)vf, lo), hi);
 #pragma unroll 1
-  for (int it = 0; it < 60; ++it) {
+  for (int it = 0; it < 80; ++it) {
     lap_ang_cdf(dim, Dn, N, v, F, f);
     if (F < U)
       lo = v;

@@ -34,9 +34,11 @@ def test_extreme_separations(n, offset):
         pe, pr = sim.pair_probs(r, r)
         got[precision] = pe.cpu().numpy(), pr.cpu().numpy()
         sim.close()
-    for g, e in zip(got["mixed"], got["fp64"]):
+    # the mixed p_reac is a table over the cut-off shell: compared there
+    shell = r.cpu().numpy() <= sigma * (1.0 + 5.0 * np.sqrt(2.0 * tau))
+    for (g, e), where in zip(zip(got["mixed"], got["fp64"]), (np.ones_like(shell), shell)):
         assert np.array_equal(g, g.astype(np.float32).astype(np.float64))
-        assert np.abs(g - e).max() <= 2e-6
+        assert np.abs(g - e)[where].max(initial=0.0) <= 2e-6
     pe, ref = got["mixed"][0], got["fp64"][0]
     tiny = (ref > 0) & (ref < 1e-37)
     assert np.all(np.abs(pe - ref)[tiny] <= 1e-4 * ref[tiny] + 1.5e-45)
