@@ -138,7 +138,7 @@ typedef struct {
                                          needing more than 127 partial waves, kappa = R' R0 / 2 tau
                                          beyond ~53, keeps the free step's direction and is counted in
                                          RD_STAT_ANGLE_FALLBACK).  RD_FP64 evaluates the series per
-                                         pair (about a millisecond of FP64 work each); RD_MIXED reads a
+                                         pair (a warp and about 60 us each, in parallel); RD_MIXED reads a
                                          per-rule table of the law built at rd_init (within 1e-4 in
                                          the law's CDF); 1 the free step's direction kept, only the
                                          length resampled */
@@ -321,8 +321,8 @@ int rd_kernel_times(rd_handle* h, int32_t cap, int32_t* n_out, char* names /* ca
  * tau = (D_A + D_B) dt / sigma^2, so large steps do not fit: the 10 uM reversible system
  * (sigma = 0.005, D_A + D_B = 2) fits at dt = 1e-5 but not at dt = 1e-4 in RD_MIXED (RD_FP64 needs
  * no tables).  No table of the angle law is built: with angle_mode 0 an RD_MIXED call evaluates
- * that law per resampled pair in FP32 (about a millisecond of one warp each), where a handle reads
- * its table, so the two agree within the FP32 angle tolerance, not bit for bit.  Inputs beyond any
+ * that law per resampled pair in FP64 (a warp and about 60 us each), where a handle reads its table,
+ * so the two agree within the FP32 angle tolerance, not bit for bit.  Inputs beyond any
  * limit are rejected with RD_EINVAL before anything is enqueued, and the outputs are left
  * untouched.
  *

@@ -8,16 +8,14 @@
 // D_n = int_0^inf e^{-tau x^2} x^{d-1} [C^ref_n(R',x) C^ref_n(R0,x) - C^abs_n(R',x) C^abs_n(R0,x)] dx,
 // with C_n(R, x) = [Z1_n(Rx) b_n(x) - Z2_n(Rx) a_n(x)] / sqrt(a_n^2 + b_n^2) from the spherical (3D)
 // or integer-order (2D, Eq. fRad) Bessel functions of the first and second kind; reflective:
-// (a, b) = x times the derivatives of (Z1, Z2) at x; absorbing: (a, b) = (Z1, Z2) at x.  The
-// functions come from their three-term recurrences (Eq. 3termBessel): the second kind upward, the
-// first kind downward from far above, normalised by its sum rule.
+// (a, b) = x times the derivatives of (Z1, Z2) at x; absorbing: (a, b) = (Z1, Z2) at x.
 //
-// One warp evaluates one pair: the lanes share the quadrature nodes (composite 16-point
-// Gauss-Legendre over x in [0, sqrt(46/tau)] in 3D, over t = sqrt(x) in 2D, with
-// 8 + ceil(sqrt(46/tau)(R'+R0)/1.5) panels), the D_n are
-// reduced across the warp and held distributed (lane l keeps D_l, D_{l+32}, ...), and the angle is
-// found by bisection of the CDF, every lane evaluating its own orders' share of each CDF value.
-// All 32 lanes must call with identical arguments.  T = double (FP64 step) or float (mixed step).
+// The FP64 step (and a mixed step without a table) evaluates the law per pair from the Laplace
+// transforms (rd_laplace.cuh).  This file holds the placement about the start separation and the mixed
+// step's table, whose nodes are built from the integrals above as they stand: the functions from their
+// three-term recurrences (Eq. 3termBessel; the second kind upward, the first kind downward from far
+// above, normalised by its sum rule), composite 16-point Gauss-Legendre over x in [0, sqrt(46/tau)] in
+// 3D, over t = sqrt(x) in 2D, with 8 + ceil(sqrt(46/tau)(R'+R0)/1.5) panels, one warp per node.
 //
 // Mixed step: the law is tabulated once per pair rule instead (FP64 build, one warp per node).  The
 // table holds, on a grid of (R0, R') and of U, the CDF value s that the exact angle has under a

@@ -677,8 +677,8 @@ static cudaError_t autotune(rd_handle* h) {
     }
   }
   // one fused launch per step or one launch per kernel (bit-identical results either way)
-  // (not with the FP64 step's exact angle pass, which can take far longer than a grid barrier
-  // waits: about a millisecond of FP64 work per pair)
+  // (not with the FP64 step's exact angle pass: a warp and about 60 us per pair, which a crowded system
+  // has tens of thousands of, against the bounded wait of a grid barrier)
   if (h->cfg.step_launch == 0 && h->L.fused_grid >= 1 && h->L.cap_particles <= kFusedMaxCapacity &&
       !(h->cfg.angle_mode == 0 && h->cfg.precision == RD_FP64)) {
     h->L.fused = !h->L.fused;

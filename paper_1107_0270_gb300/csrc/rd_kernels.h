@@ -173,10 +173,12 @@ struct FptArgs {
 // Where a pair moves on.  A lane draws one attempt at a time, about 3000 cycles each once the other lanes
 // have finished, so a large first budget is a long tail with few lanes busy; a small one sends pairs to a
 // warp that would have finished soon.  2^20 pairs, 10 levels, FP32 / FP64: 256, 4352, 32768 2.27 / 41 ms;
-// 64, 1024, 16384 1.38 / 29; 48, 512, 8192 1.30 / 27.8; 24, 384, 4096 1.38 / 31.
+// 64, 1024, 32768 1.53 / 32; 48, 512, 36816 1.41 / 31.7; 24, 384, 4096 1.38 / 31.  (With 8192 in the block
+// phase 1.30 / 27.8, but the grid phase's FP32 attempt differs from the other phases' in the last bit now
+// and then, so a pair must not reach it sooner than at 37 376 draws, where it always did.)
 constexpr uint32_t kFptBudget = 48;         // draws per pair in the lane-per-pair phase
 constexpr uint32_t kFptWarpBudget = 512;    // further draws before the block-per-pair phase
-constexpr uint32_t kFptBlockBudget = 8192;  // further draws before the grid phase
+constexpr uint32_t kFptBlockBudget = 36816; // further draws before the grid phase
 constexpr int kFptBlockThreads = 512;       // threads per pair in the block-per-pair phase
 constexpr int kFptGridThreads = 256;        // threads per block (and attempts per chunk) of the grid phase
 constexpr uint32_t kFptGridGroups = 4;      // block groups of the grid phase, each searching its own pairs
