@@ -607,7 +607,8 @@ __device__ __forceinline__ void ph_sweep(const DevParams* Pp, DevCtl* ctl,
     if constexpr (sizeof(T) == 8) {
       // The cut-off is decided in FP64; then a pair fires only if its draw lies below p_enc, so the
       // draw is compared with p_enc in FP32 (3D; in 2D with p_enc's closed bound) plus a margin over
-      // its rounding, and only the pairs below that, or as close to contact, take the FP64 evaluation.
+      // its rounding (p_enc_screen), and only the pairs below that, or so close to contact that FP32
+      // cannot tell which side of it they are on, take the FP64 evaluation.
       const double r0x = min_image(b0.x - a0.x, rep.L, rep.half_L);
       const double r0y = min_image(b0.y - a0.y, rep.L, rep.half_L);
       const double r0z = dim == 3 ? min_image(b0.z - a0.z, rep.L, rep.half_L) : 0.0;

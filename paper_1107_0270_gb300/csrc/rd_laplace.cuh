@@ -388,18 +388,24 @@ __device__ __noinline__ double lap_p_enc2_warp(double R, double R0, double tau) 
 }
 
 // FP32 value that the FP64 step's encounter draw must lie below for the pair to need its exact p_enc,
-// from the contact distances d = R - 1 > 0 and d0 = R0 - 1 rounded to FP32 (errors about 1e-6).
+// from the contact distances d = R - 1 > 0 and d0 = R0 - 1 computed in FP32.
 // 3D: the FP32 closed form.  2D: a closed upper bound: u(R) = sqrt(R) g obeys the 1D diffusion equation
 // plus the growth term u / 4R^2, so g_abs is at least the 1D absorbing kernel over sqrt(R R0),
 //   1 - p_enc >= (1 - e^{-d d0/tau}) / m,  m = sqrt(2 pi z) e^{-z} I0(z), z = R R0/2tau.
-// The margin of 1e-4 is far above the rounding of either.
+// Margin: with e = 2^-24, the squared length, the root, the contact radius and its reciprocal leave
+// each distance within 6e (1 + d) of its value, so the exponent x = d d0 / tau is within
+// 6e ((d + d0)/tau + 2x) and p <= e^{-x} within that times p, which grows like 1/sqrt(tau): at
+// tau = 1e-7 up to 1e-3.  The first part of the margin is 5e-7 (d + d0)/tau (6e = 3.6e-7); the 1e-4 are
+// far above the rest: 2x e^{-x} 6e < 3e-7 and a few e of the factors (in 2D also where m < 1, since
+// x e^{-x}/m <= (1 - e^{-x})/m <= 1, and (d + d0)/(tau m) < 12 there).
 __device__ __forceinline__ float p_enc_screen(int dim, float d, float d0, float inv_tau) {
   if (d0 <= 0.0f) return 2.0f;
-  if (dim == 3) return p_enc3_f(d, d0, inv_tau) + 1e-4f;
+  const float margin = 1e-4f + 5e-7f * (d + d0) * inv_tau;
+  if (dim == 3) return p_enc3_f(d, d0, inv_tau) + margin;
   const float z = (1.0f + d) * (1.0f + d0) * 0.5f * inv_tau;
   const float m = z < 40.0f ? sqrtf(6.2831853f * z) * expf(-z) * cyl_bessel_i0f(z)
                             : 1.0f + 0.125f / z + 0.0703125f / (z * z) + 0.0732422f / (z * z * z);
-  return 1.0f + expm1f(-d * d0 * inv_tau) / m + 1e-4f;
+  return 1.0f + expm1f(-d * d0 * inv_tau) / m + margin;
 }
 
 // Eq. (psurv_radII) in 2D.  Warp-collective.
