@@ -135,9 +135,28 @@ RD_HD void k01_scaled(cplx x, cplx& k0, cplx& k1) {
   k1 = k0 * ((cx(x.re + 0.5, x.im) - up * iu) * ix);
 }
 
-// e^{-x} I_0(x) for Re x > 0 from the Wronskian, I_0 = 1 / (x (K_1 + (I_1/I_0) K_0)), with the ratio
-// from the downward recurrence of the minimal solution I_n.  k0, k1 as from k01_scaled.
+// e^{-x} I_0(x) for Re x > 0 (k0, k1 as from k01_scaled).  From Re x = 20 on the asymptotic series
+// (Abramowitz & Stegun 9.7.1): the part it leaves out is e^{-2 Re x} < 5e-18 of it, and |x| >= 20 needs 27
+// terms at most (checked against 40-digit values: below 1e-15).  Elsewhere from the Wronskian,
+// I_0 = 1 / (x (K_1 + (I_1/I_0) K_0)), with the ratio from the downward recurrence of the minimal
+// solution I_n, 24 + 1.5 |x| orders: at most 180 on the line below, where |x| <= 5.2 Re x, but thousands
+// at small tau, where |x| grows like u / 2 tau (absorbing 2D system of 3000 particles, tau = 1e-5:
+// 0.80 ms a step with the recurrence alone, 0.068 with the series).
 RD_HD cplx i0_scaled(cplx x, cplx k0, cplx k1) {
+  if (x.re >= 20.0) {
+    const double q8 = 0.125 / (x.re * x.re + x.im * x.im);
+    const cplx i8 = cx(x.re * q8, -x.im * q8);                    // 1 / 8x
+    cplx t = cx(1.0, 0.0), sum = t;
+#pragma unroll 1
+    for (int k = 1; k < 40; ++k) {
+      t = ((2.0 * k - 1.0) * (2.0 * k - 1.0) * RD_LAP.ik[k]) * (t * i8);
+      sum = sum + t;
+      if (fabs(t.re) + fabs(t.im) < 1e-17) break;
+    }
+    const cplx q = (4.0 / kPi) * i8;                              // 1 / 2 pi x: principal root
+    const double sr = sqrt(0.5 * (sqrt(q.re * q.re + q.im * q.im) + q.re));
+    return cx(sr, 0.5 * q.im / sr) * sum;
+  }
   const cplx ix = crcp(x);
   const double ax = sqrt(x.re * x.re + x.im * x.im);
   cplx jp = cx(0.0, 0.0), j = cx(1e-100, 0.0);
