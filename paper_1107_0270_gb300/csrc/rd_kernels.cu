@@ -1615,7 +1615,8 @@ __device__ __forceinline__ void replica_table(int n_replicas, const RepDev* reps
 }
 
 // One accepted pair or one decay of this step (item q of the combined list), by one thread, or (FP64
-// step in 2D) by a warp whose lanes share the law's nodes, lead marking the lane that writes.
+// step in 2D) by a warp whose lanes share the law's nodes, lead marking the lane that writes.  spread: the
+// step's items are on many blocks.
 template <class T>
 __device__ __noinline__ void resolve_item(const DevParams& P, const RepDev* reps,
                                              const FiredPair* fired, const uint32_t* fstate,
@@ -1627,7 +1628,7 @@ __device__ __noinline__ void resolve_item(const DevParams& P, const RepDev* reps
                                              unsigned long long& n_react, unsigned long long& n_res,
                                              unsigned long long& n_rec, unsigned long long& n_near,
                                              DevCtl* ctl, AngJob* jobs, uint32_t job_cap, uint2* events,
-                                             bool lead) {
+                                             bool spread, bool lead) {
   if constexpr (sizeof(T) == 8) {
     if (pair)
       resolve_pair<T>(P, reps, fired, fstate, idx, step, x0, x1, status, prodpos, n_react, n_res, n_near, ctl, jobs,
@@ -1651,7 +1652,16 @@ __device__ __noinline__ void resolve_item(const DevParams& P, const RepDev* reps
     const uint32_t np = (st >> ST_NPROD_SHIFT) & 3u;
     if (np) atomicAdd(&rep_prod[r], np);
     // the consumed particles (and the products of their owner) for the compaction
-    const uint32_t k = pair ? 2u : 1u, e = atomicAdd(&ctl->n_ev, k);
+    // (items on many blocks: one atomic per warp, since in a step that consumes millions all go to one counter)
+    const uint32_t k = pair ? 2u : 1u;
+    uint32_t e = 0;
+    if (spread) {
+      const unsigned act = __activemask(), two = __ballot_sync(act, pair), below = (1u << (threadIdx.x & 31)) - 1u;
+      if ((act & below) == 0u) e = atomicAdd(&ctl->n_ev, (uint32_t)(__popc(act) + __popc(two)));
+      e = __shfl_sync(act, e, __ffs(act) - 1) + (uint32_t)(__popc(act & below) + __popc(two & below));
+    } else {
+      e = atomicAdd(&ctl->n_ev, k);
+    }
     if (e + k <= kMaxEvents) {
       events[e] = make_uint2(owner, np);
       if (pair) events[e + 1] = make_uint2(fired[idx].ib, 0u);
@@ -1714,7 +1724,7 @@ __device__ __forceinline__ void ph_match_resolve(
     for (uint32_t q = q0; q < n_triv + nd; q += nblk * (by_warp ? wpb : blockDim.x)) {
       const bool pair = q < n_triv;
       resolve_item<T>(P, reps, fired, fstate, pair, pair ? accepted[q] : decay_list[q - n_triv], step, x0, x1, id,
-                      status, prodpos, rep_cons, rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap, events, lead);
+                      status, prodpos, rep_cons, rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap, events, true, lead);
     }
   }
   if (nc > 0 && !multi && nc <= min(P.match_smem_max, (uint32_t)kMatchSmemPairs) && blockIdx.x == 0) {
@@ -1725,7 +1735,7 @@ __device__ __forceinline__ void ph_match_resolve(
       const uint32_t n_acc = n_triv + *(volatile uint32_t*)&ctl->n_round_acc;
       for (uint32_t q = n_triv + (by_warp ? wid : threadIdx.x); q < n_acc; q += by_warp ? wpb : blockDim.x)
         resolve_item<T>(P, reps, fired, fstate, true, accepted[q], step, x0, x1, id, status, prodpos, rep_cons,
-                        rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap, events, lead);
+                        rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap, events, true, lead);
     }
   } else if (nc > 0 && (multi ? blockIdx.x < nrb : blockIdx.x == 0)) {
     const uint32_t nthr = multi ? nrb * blockDim.x : blockDim.x;
@@ -1865,7 +1875,7 @@ __device__ __forceinline__ void ph_match_resolve(
       for (uint32_t q = first + q0; q < last; q += by_warp ? nthr >> 5 : nthr) {
         const bool pair = q < n_acc;
         resolve_item<T>(P, reps, fired, fstate, pair, pair ? accepted[q] : decay_list[q - n_acc], step, x0, x1, id,
-                        status, prodpos, rep_cons, rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap, events, lead);
+                        status, prodpos, rep_cons, rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap, events, true, lead);
       }
     }
   }
@@ -1935,7 +1945,7 @@ __device__ __forceinline__ void match_resolve_few(
   unsigned long long n_react = 0, n_res = 0, n_near = 0, n_rec = 0;
   if (mine)
     resolve_item<T>(P, reps, fired, fstate, q < nf, q < nf ? q : decay_list[q - nf], step, x0, x1, id, status, prodpos,
-                    rep_cons, rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap, events, true);
+                    rep_cons, rep_prod, n_react, n_res, n_rec, n_near, ctl, jobs, job_cap, events, false, true);
   if (n_react) atomicAdd(&ctl->stats[RD_STAT_REACTIONS], n_react);
   if (n_res) atomicAdd(&ctl->stats[RD_STAT_RESAMPLED], n_res);
   if (n_rec) atomicAdd(&ctl->stats[RD_STAT_RECOMBINED], n_rec);
@@ -2065,17 +2075,45 @@ __global__ void __launch_bounds__(256, 2) k_angles(const DevParams* __restrict__
   ph_angles<T>(Pp, ctl, reps, jobs, job_cap, x1, prodpos, blockIdx.x, gridDim.x);
 }
 
-// Count of a (replica, species) key: atomically up or down by one.  Only particles that leave or join
-// are counted; the counts carry over from step to step.
-__device__ __forceinline__ void count_event(uint32_t wb, int ns, bool up, unsigned long long* counts, int32_t* s_tot) {
-  const unsigned long long one = 1ull;
-  atomicAdd(&counts[(size_t)(wb >> 8) * ns + (wb & 0xFFu)], up ? one : ~0ull);
-  atomicAdd(&s_tot[wb & 0xFFu], up ? 1 : -1);
+constexpr uint32_t kNoKey = 0xFFFFFFFFu;
+
+// Counts the active lanes' (replica, species) words up or down, lanes of one word together: replica
+// r_blk into the block's own s_rep, others into the counts and the block's species totals.  Only
+// particles that leave or join are counted; the counts carry over from step to step.  (One atomic a
+// particle: 885 us where 1e6 of 2e6 particles decay, 65 this way.)
+__device__ __forceinline__ void count_events(uint32_t wb, int ns, bool up, uint32_t r_blk, unsigned long long* counts,
+                                             int32_t* s_rep, int32_t* s_tot) {
+  const unsigned peers = __match_any_sync(__activemask(), wb);
+  if ((int)(threadIdx.x & 31) != __ffs(peers) - 1) return;
+  const int d = up ? __popc(peers) : -__popc(peers);
+  if ((wb >> 8) == r_blk) {
+    atomicAdd(&s_rep[wb & 0xFFu], d);
+  } else {
+    atomicAdd(&counts[(size_t)(wb >> 8) * ns + (wb & 0xFFu)], (unsigned long long)(long long)d);
+    atomicAdd(&s_tot[wb & 0xFFu], d);
+  }
+}
+// One by one (the event list's; the block that ends a step waits for every cache line of instructions it
+// has to fetch, and the joint form above cost 0.15 us of a 26 us step there): ups and downs of a species,
+// and with several replicas the counts.
+__device__ __forceinline__ void count_event(uint32_t wb, int ns, bool up, bool one, unsigned long long* counts,
+                                            int32_t* s_rep, int32_t* s_tot) {
+  atomicAdd(up ? &s_tot[wb & 0xFFu] : &s_rep[wb & 0xFFu], 1);
+  if (!one) atomicAdd(&counts[(size_t)(wb >> 8) * ns + (wb & 0xFFu)], up ? 1ull : ~0ull);
+}
+// The block's own counts into the global ones and its species totals (between block barriers).
+__device__ __forceinline__ void flush_counts(int ns, uint32_t r_blk, unsigned long long* counts, int32_t* s_rep,
+                                             int32_t* s_tot) {
+  if (threadIdx.x < (unsigned)ns && s_rep[threadIdx.x]) {
+    const int32_t d = s_rep[threadIdx.x];
+    atomicAdd(&counts[(size_t)r_blk * ns + threadIdx.x], (unsigned long long)(long long)d);
+    s_tot[threadIdx.x] += d;
+    s_rep[threadIdx.x] = 0;
+  }
 }
 
 // Per-warp aggregated count: lanes holding the same (replica, species) key add once.  Called by all
 // 32 lanes of a converged warp; key kNoKey is skipped.
-constexpr uint32_t kNoKey = 0xFFFFFFFFu;
 __device__ __forceinline__ void count_key(uint32_t key, unsigned long long* counts) {
   const unsigned peers = __match_any_sync(0xFFFFFFFFu, key);
   if (key != kNoKey && (int)(threadIdx.x & 31) == __ffs(peers) - 1)
@@ -2112,7 +2150,7 @@ __device__ __forceinline__ void species_totals(const unsigned long long* counts,
 // ================================================================================================
 // Events of a tile up to which every particle looks through them; above, the tile sums marks once (the
 // compaction of 4000 particles that all decay, mixed: 250 us with every particle looking through 2048
-// events, 20 with the sums; at 20 events a tile 8 either way).
+// events, 14 with the sums; at 20 events a tile 8 either way).
 constexpr uint32_t kTileEvents = 24;
 
 // A mark per particle of the tile (consumed, products << 16) behind the list of its m events, and the
@@ -2157,11 +2195,14 @@ __device__ __forceinline__ void ph_compact(const DevParams* Pp, DevCtl* ctl,
   __shared__ uint32_t s_tile;
   __shared__ unsigned long long s_prefix;
   __shared__ bool s_last;
-  __shared__ int32_t s_tot[kMaxSpecies];
+  __shared__ int32_t s_tot[kMaxSpecies], s_rep[kMaxSpecies];
   __shared__ uint32_t s_before[2], s_inside;
   const DevParams& P = *Pp;
-  // the first tile's loads go out beside those of the control block (four passes at most)
-  constexpr int kAhead = kPasses < 4 ? kPasses : 4;
+  // passes whose loads are in flight at once (128 bytes a thread at most).  The 1024-thread tiles of small
+  // systems issue the first tile's beside those of the control block; the others once the event list is
+  // known to be used (the status scan's form reads the particles itself).
+  constexpr int kMaxAhead = sizeof(T) == 8 ? 2 : 4, kAhead = kPasses < kMaxAhead ? kPasses : kMaxAhead;
+  constexpr bool kEager = kCompactThreads == 1024;
   typename V4<T>::type q[kAhead];
   uint32_t idv[kAhead];
   auto load_passes = [&](const int64_t t0, const int first, const uint32_t end) {
@@ -2174,7 +2215,7 @@ __device__ __forceinline__ void ph_compact(const DevParams* Pp, DevCtl* ctl,
       }
     }
   };
-  load_passes((int64_t)bid * kTile, 0, cap);
+  if (kEager) load_passes((int64_t)bid * kTile, 0, cap);
   const int ns = P.n_species;
   const uint32_t n = ctl->n, n_ev = ctl->n_ev;
   // a single replica: its placement follows from the step's tallies directly
@@ -2189,7 +2230,8 @@ __device__ __forceinline__ void ph_compact(const DevParams* Pp, DevCtl* ctl,
   const bool fail = ctl->status != 0 || (unsigned long long)n_new > (unsigned long long)P.cap_particles;
   const bool few = !fail && n_ev <= kMaxEvents;
   const uint32_t ntiles = (uint32_t)(((int64_t)n + kTile - 1) / kTile);
-  if (threadIdx.x < kMaxSpecies) s_tot[threadIdx.x] = 0;
+  if (threadIdx.x < kMaxSpecies) s_tot[threadIdx.x] = s_rep[threadIdx.x] = 0;
+  uint32_t r_blk = kNoKey;      // replica whose counts the block gathers in s_rep
   // the products of owner i, P_i products before it
   auto place_products = [&](uint32_t i, uint32_t np, uint32_t P_i, const RepX& rx, uint32_t r) {
     for (uint32_t k = 0; k < np; ++k) {
@@ -2197,7 +2239,7 @@ __device__ __forceinline__ void ph_compact(const DevParams* Pp, DevCtl* ctl,
       const auto pp = prodpos[2 * (size_t)i + k];
       xo[o] = pp;
       ido[o] = reps[r].next_id + (P_i - rx.p_beg) + k;
-      if (!few) count_event(w_bits(pp.w), ns, true, counts, s_tot);
+      if (!few) count_events(w_bits(pp.w), ns, true, r_blk, counts, s_rep, s_tot);
     }
   };
   if (few) {
@@ -2217,10 +2259,10 @@ __device__ __forceinline__ void ph_compact(const DevParams* Pp, DevCtl* ctl,
     };
     for (uint32_t tile = bid; tile < ntiles; tile += nblk) {
       const int64_t t0 = (int64_t)tile * kTile;
-      __syncthreads();
+      if (tile != bid) __syncthreads();
       if (threadIdx.x == 0) s_before[0] = s_before[1] = s_inside = 0u;
       __syncthreads();
-      if (tile != bid) load_passes(t0, 0, n);
+      if (!kEager || tile != bid) load_passes(t0, 0, n);
       uint32_t cb = 0, pb = 0;
       for (uint32_t e = threadIdx.x; e < n_ev; e += kCompactThreads) {
         const uint2 v = events[e];
@@ -2275,12 +2317,14 @@ __device__ __forceinline__ void ph_compact(const DevParams* Pp, DevCtl* ctl,
     // tiles by ticket, so that every tile's predecessors are taken before it (look-back order)
     for (;;) {
       __syncthreads();
+      flush_counts(ns, r_blk, counts, s_rep, s_tot);
       if (threadIdx.x == 0) s_tile = atomicAdd(&ctl->tile_ctr[1], 1u);
       __syncthreads();
       const uint32_t tile = s_tile;
       if (tile >= ntiles) break;
       const int64_t t0 = (int64_t)tile * kTile;
       if (!fail) {
+        r_blk = w_bits(x1[t0].w) >> 8;      // particles are ordered by replica: most of the tile's belong to it
         // blocked arrangement for the scan: each thread owns kCompactItems consecutive particles
         const int64_t base = t0 + (int64_t)threadIdx.x * kCompactItems;
         unsigned long long v[kCompactItems], ex[kCompactItems], run = 0;
@@ -2309,7 +2353,7 @@ __device__ __forceinline__ void ph_compact(const DevParams* Pp, DevCtl* ctl,
         __syncthreads();
       }
       // striped placement (coalesced), one particle per thread per pass
-#pragma unroll
+#pragma unroll 2
       for (int ps = 0; ps < kPasses; ++ps) {
         const int j = threadIdx.x + ps * kCompactThreads;
         const int64_t i = t0 + j;
@@ -2330,7 +2374,7 @@ __device__ __forceinline__ void ph_compact(const DevParams* Pp, DevCtl* ctl,
           xo[o] = q;
           ido[o] = id[i];
         } else {
-          count_event(wb, ns, false, counts, s_tot);
+          count_events(wb, ns, false, r_blk, counts, s_rep, s_tot);
         }
         place_products((uint32_t)i, (st >> ST_NPROD_SHIFT) & 3u, P_i, rx, r);
       }
@@ -2348,8 +2392,9 @@ __device__ __forceinline__ void ph_compact(const DevParams* Pp, DevCtl* ctl,
   if (few) {
     for (uint32_t e = threadIdx.x; e < n_ev; e += blockDim.x) {
       const uint2 v = events[e];
-      count_event(w_bits(x0[v.x].w), ns, false, counts, s_tot);
-      for (uint32_t k = 0; k < v.y; ++k) count_event(w_bits(prodpos[2 * (size_t)v.x + k].w), ns, true, counts, s_tot);
+      count_event(w_bits(x0[v.x].w), ns, false, one, counts, s_rep, s_tot);
+      for (uint32_t k = 0; k < v.y; ++k)
+        count_event(w_bits(prodpos[2 * (size_t)v.x + k].w), ns, true, one, counts, s_rep, s_tot);
     }
   } else {
     __threadfence();
@@ -2368,7 +2413,9 @@ __device__ __forceinline__ void ph_compact(const DevParams* Pp, DevCtl* ctl,
   __syncthreads();
   // per-step totals over replicas of every species (ring buffer indexed by the new step)
   if (!fail && threadIdx.x < (unsigned)ns) {
-    const long long t = *(volatile long long*)&ctl->tot[threadIdx.x] + (few ? (long long)s_tot[threadIdx.x] : 0ll);
+    const long long d = few ? (long long)(s_tot[threadIdx.x] - s_rep[threadIdx.x]) : 0ll;
+    if (one && d) atomicAdd(&counts[threadIdx.x], (unsigned long long)d);     // (with several: counted above)
+    const long long t = *(volatile long long*)&ctl->tot[threadIdx.x] + d;
     ctl->tot[threadIdx.x] = t;
     if (history_len > 0) history[(size_t)((ctl->step + 1u) % (uint32_t)history_len) * ns + threadIdx.x] = t;
   }

@@ -117,3 +117,8 @@ def exchanging(n, kdt, replicas=None):
 def test_a_tile_full_of_events_costs_a_scan_not_a_search():
     # every particle looking through its tile's events: 250 us against 8 without events
     assert compaction_us(exchanging(4000, 30.0)) <= 6.0 * compaction_us(exchanging(4000, 1e-9))
+
+
+def test_counting_many_events_is_not_one_atomic_each():
+    # an atomic on a species' one count per particle: 148 us against 12 without events
+    assert compaction_us(exchanging(400_000, 0.5)) <= 5.0 * compaction_us(exchanging(400_000, 1e-9))
