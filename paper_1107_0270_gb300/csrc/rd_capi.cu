@@ -416,6 +416,8 @@ static bool build_2d(const rd_config& c, DevParams& hp, Alloc alloc) {
 // FP32 lookup tables of the mixed step (p_reac in 2D and 3D; F = p_enc e^{d d0/tau} and
 // -ln(tail) in 2D), spacing 0.025 min(sqrt(tau), 1) over d0 up to the cut-off and d up to the propagator's
 // support (d0 + 13 sqrt(tau)), built in FP64 on the device.
+constexpr size_t kMaxPairedRows = (size_t)64 << 20;
+
 template <class Alloc>
 static cudaError_t build_tables(rd_handle* h, Alloc alloc) {
   const rd_config& c = h->cfg;
@@ -434,11 +436,9 @@ static cudaError_t build_tables(rd_handle* h, Alloc alloc) {
       const size_t bytes = (size_t)n0 * m1 * sizeof(float);
       float* t = (float*)alloc(bytes);
       float4* q4 = (float4*)alloc(4 * bytes);
-      float4* q8 = kind == 0 ? (float4*)alloc(8 * bytes) : nullptr;     // rd_pair_probs reads p_reac in pairs of rows
       double* tot = (double*)alloc((size_t)n0 * sizeof(double));
-      if (!t || !q4 || !tot || (kind == 0 && !q8)) return cudaErrorMemoryAllocation;
-      launch_build_table(h->L.P, k, kind, t, q4, q8, n0, m1, hstep, h1, tot, fwd, device_sms(), h->stream);
-      T.q2 = q8;
+      if (!t || !q4 || !tot) return cudaErrorMemoryAllocation;
+      launch_build_table(h->L.P, k, kind, t, q4, n0, m1, hstep, h1, tot, fwd, device_sms(), h->stream);
       T.v = t;
       T.q = q4;
       T.n0 = n0;
@@ -485,7 +485,24 @@ static cudaError_t build_tables(rd_handle* h, Alloc alloc) {
     }
     if (e != cudaSuccess) return e;
   }
-  cudaError_t e = cudaStreamSynchronize(h->stream);
+  // Paired rows of the 3D p_reac tables, which rd_pair_probs reads in half as many loads (2^25 pairs 451 ->
+  // 367 us, the same values).  They take more than the table itself and nothing else needs them: built
+  // last, up to 64 MB a rule (tau of about 9; beyond, the table is far larger than the L2 keeps anyway),
+  // and left out where the allocator has no room.
+  for (int k = 0; k < c.n_pairs && c.dim == 3; ++k) {
+    Tab2& T = h->hp.pairs[k].tab_preac;
+    const size_t bytes = (size_t)T.n0 * T.n1 * 2 * sizeof(float4);
+    if (!T.q || bytes > kMaxPairedRows) continue;
+    float4* q2 = (float4*)alloc(bytes);
+    if (!q2) {
+      cudaGetLastError();
+      continue;
+    }
+    launch_table_pairs(T.q, T.n0, T.n1, q2, device_sms(), h->stream);
+    T.q2 = q2;
+  }
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return e;
   return cudaMemcpy((void*)h->L.P, &h->hp, sizeof(DevParams), cudaMemcpyHostToDevice);
 }
@@ -1184,7 +1201,8 @@ int rd_pair_probs(rd_handle* h, int32_t rule, const double* r0, const double* r,
   if (h->cfg.pairs[rule].bc == RD_BC_NONE) return RD_EINVAL;
   if (n == 0) return RD_OK;
   launch_pair_probs(h->L.P, rule, r0, r, n, p_enc, p_reac, h->L.max_grid,
-                    h->cfg.precision == RD_MIXED && h->cfg.dim == 3, h->stream);
+                    h->cfg.precision == RD_MIXED && h->cfg.dim == 3, h->hp.pairs[rule].tab_preac.q2 != nullptr,
+                    h->stream);
   RD_CUDA(cudaGetLastError());
   return RD_OK;
 }
@@ -1668,7 +1686,7 @@ extern "C" int rd_step_static(const rd_config* cfg, void* stream, int64_t n, con
   }
   RD_CUDA(cudaMemcpyAsync((void*)L.P, &hp0, sizeof(DevParams), cudaMemcpyHostToDevice, s));
   for (const TableJob& j : jobs)
-    launch_build_table(L.P, j.rule, j.kind, j.t, j.q4, nullptr, j.n0, j.m1, j.hstep, j.h1, j.tot, nullptr, device_sms(), s);
+    launch_build_table(L.P, j.rule, j.kind, j.t, j.q4, j.n0, j.m1, j.hstep, j.h1, j.tot, nullptr, device_sms(), s);
   if (!jobs.empty()) RD_CUDA(cudaMemcpyAsync((void*)L.P, &tmp.hp, sizeof(DevParams), cudaMemcpyHostToDevice, s));
   RD_CUDA(cudaMemcpyAsync(L.reps, &rep, sizeof rep, cudaMemcpyHostToDevice, s));
   RD_CUDA(cudaMemcpyAsync(L.ctl, &ctl, sizeof ctl, cudaMemcpyHostToDevice, s));

@@ -2529,8 +2529,9 @@ __global__ void k_count(const DevParams* __restrict__ Pp, const DevCtl* __restri
 
 // Standalone per-pair probabilities (rd_pair_probs).
 // p_enc and p_reac of one pair at start / end separations a, b (um); kMixed3D: the mixed step in
-// 3D (no FP64 or 2D branch compiled, which keeps the streaming kernel's register count low).
-template <bool kMixed3D>
+// 3D (no FP64 or 2D branch compiled, which keeps the streaming kernel's register count low); kPaired: its
+// p_reac table has the paired rows.
+template <bool kMixed3D, bool kPaired>
 __device__ __forceinline__ void pair_probs_one(const DevParams& P, const PairDev& pr, double a, double b, double& pe,
                                                double& prc, bool want_enc, bool want_reac) {
   // mixed: the separations rounded once to FP32 and scaled there (FP64 arithmetic runs at 1/64 of
@@ -2558,7 +2559,7 @@ __device__ __forceinline__ void pair_probs_one(const DevParams& P, const PairDev
     double v = pr.bc == RD_BC_ABS ? 1.0 : 0.0;
     if (pr.bc == RD_BC_RAD) {
       if (kMixed3D)
-        v = widen(p_reac_tab2(pr, d, d0));
+        v = widen(kPaired ? p_reac_tab2(pr, d, d0) : p_reac_tab(pr, d, d0));
       else
         v = P.precision == RD_MIXED ? (double)p_reac_tab(pr, d, d0) : p_reac_dim(P, pr, b / pr.sigma, a / pr.sigma);
     }
@@ -2569,7 +2570,7 @@ __device__ __forceinline__ void pair_probs_one(const DevParams& P, const PairDev
 // Standalone pair probabilities (streaming).  With 16-byte aligned arrays each thread takes four
 // consecutive pairs per pass through 16-byte loads and stores (more bytes in flight per thread);
 // the remainder, or unaligned arrays, one pair per thread.
-template <bool kMixed3D>
+template <bool kMixed3D, bool kPaired>
 __global__ void k_pair_probs(const DevParams* __restrict__ Pp, int rule, const double* __restrict__ r0,
                              const double* __restrict__ r, int64_t n, double* __restrict__ p_enc,
                              double* __restrict__ p_reac) {
@@ -2587,10 +2588,10 @@ __global__ void k_pair_probs(const DevParams* __restrict__ Pp, int rule, const d
       const double2 b01 = __ldcs(reinterpret_cast<const double2*>(r) + 2 * q);
       const double2 b23 = __ldcs(reinterpret_cast<const double2*>(r) + 2 * q + 1);
       double e[4] = {0, 0, 0, 0}, c[4] = {0, 0, 0, 0};
-      pair_probs_one<kMixed3D>(P, pr, a01.x, b01.x, e[0], c[0], we, wr);
-      pair_probs_one<kMixed3D>(P, pr, a01.y, b01.y, e[1], c[1], we, wr);
-      pair_probs_one<kMixed3D>(P, pr, a23.x, b23.x, e[2], c[2], we, wr);
-      pair_probs_one<kMixed3D>(P, pr, a23.y, b23.y, e[3], c[3], we, wr);
+      pair_probs_one<kMixed3D, kPaired>(P, pr, a01.x, b01.x, e[0], c[0], we, wr);
+      pair_probs_one<kMixed3D, kPaired>(P, pr, a01.y, b01.y, e[1], c[1], we, wr);
+      pair_probs_one<kMixed3D, kPaired>(P, pr, a23.x, b23.x, e[2], c[2], we, wr);
+      pair_probs_one<kMixed3D, kPaired>(P, pr, a23.y, b23.y, e[3], c[3], we, wr);
       if (we) {
         __stcs(reinterpret_cast<double2*>(p_enc) + 2 * q, make_double2(e[0], e[1]));
         __stcs(reinterpret_cast<double2*>(p_enc) + 2 * q + 1, make_double2(e[2], e[3]));
@@ -2604,7 +2605,7 @@ __global__ void k_pair_probs(const DevParams* __restrict__ Pp, int rule, const d
   }
   for (int64_t k = done + tid; k < n; k += stride) {
     double e = 0.0, c = 0.0;
-    pair_probs_one<kMixed3D>(P, pr, r0[k], r[k], e, c, we, wr);
+    pair_probs_one<kMixed3D, kPaired>(P, pr, r0[k], r[k], e, c, we, wr);
     if (we) p_enc[k] = e;
     if (wr) p_reac[k] = c;
   }
@@ -2745,19 +2746,28 @@ __global__ void k_table_ghost_row(float* __restrict__ T, int n1) {
 }
 
 // quad layout of a finished table: q[i n1 + j] = (v[i n1 + j-1], .., v[i n1 + j+2]), zero off the ends
-__global__ void k_table_quads(const float* __restrict__ T, int n0, int n1, float4* __restrict__ Q,
-                              float4* __restrict__ Q2) {
+__global__ void k_table_quads(const float* __restrict__ T, int n0, int n1, float4* __restrict__ Q) {
   const int64_t total = (int64_t)n0 * n1;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total; k += (int64_t)gridDim.x * blockDim.x) {
     const int j = (int)(k % n1);
     float4 q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (j >= 1 && j + 2 < n1) q = make_float4(T[k - 1], T[k], T[k + 1], T[k + 2]);
     Q[k] = q;
-    if (Q2) {
-      Q2[2 * k] = q;
-      if (k >= n1) Q2[2 * (k - n1) + 1] = q;
-    }
   }
+}
+
+// paired rows of a table's quads: q2[2 (i n1 + j)] = q[i n1 + j], q[(i+1) n1 + j] (the last row's partner is
+// not read)
+__global__ void k_table_pairs(const float4* __restrict__ Q, int n0, int n1, float4* __restrict__ Q2) {
+  const int64_t total = (int64_t)n0 * n1;
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total; k += (int64_t)gridDim.x * blockDim.x) {
+    Q2[2 * k] = Q[k];
+    Q2[2 * k + 1] = Q[k + n1 < total ? k + n1 : k];
+  }
+}
+
+void launch_table_pairs(const float4* quad, int n0, int n1, float4* quad2, int device_sms, cudaStream_t s) {
+  k_table_pairs<<<device_sms * 8, 128, 0, s>>>(quad, n0, n1, quad2);
 }
 
 // 2D inverse table from a finished forward -ln(tail) table: at each node (d0, t) the V where the
@@ -2781,7 +2791,7 @@ __global__ void k_build_inverse2(Tab2 fwd, float* __restrict__ out, int n0, int 
   }
 }
 
-void launch_build_table(const DevParams* P, int rule, int kind, float* out, float4* quad, float4* quad2, int n0, int n1, double h,
+void launch_build_table(const DevParams* P, int rule, int kind, float* out, float4* quad, int n0, int n1, double h,
                         double h1, double* tot, const Tab2* fwd, int device_sms, cudaStream_t s) {
   if (kind == 2) k_tail_totals<<<(n0 + 63) / 64, 64, 0, s>>>(P, rule, n0, h, tot);
   const int64_t total = (int64_t)n0 * n1;
@@ -2792,7 +2802,7 @@ void launch_build_table(const DevParams* P, int rule, int kind, float* out, floa
     k_build_table<<<G, 128, 0, s>>>(P, rule, kind, out, n0, n1, h, h1, tot);
   k_table_ghosts<<<(n0 + 255) / 256, 256, 0, s>>>(out, n0, n1);
   k_table_ghost_row<<<(n1 + 255) / 256, 256, 0, s>>>(out, n1);
-  k_table_quads<<<G, 128, 0, s>>>(out, n0, n1, quad, quad2);
+  k_table_quads<<<G, 128, 0, s>>>(out, n0, n1, quad);
 }
 
 // ================================================================================================
@@ -3225,11 +3235,12 @@ void launch_count(const StepLaunch& L, cudaStream_t s) {
 }
 
 void launch_pair_probs(const DevParams* P, int rule, const double* r0, const double* r, int64_t n, double* pe,
-                       double* pr, int max_grid, bool mixed3d, cudaStream_t s) {
-  if (mixed3d)
-    k_pair_probs<true><<<grid_for(n, 256, max_grid), 256, 0, s>>>(P, rule, r0, r, n, pe, pr);
+                       double* pr, int max_grid, bool mixed3d, bool paired, cudaStream_t s) {
+  auto go = [&](auto kernel) { kernel<<<grid_for(n, 256, max_grid), 256, 0, s>>>(P, rule, r0, r, n, pe, pr); };
+  if (!mixed3d)
+    go(k_pair_probs<false, false>);
   else
-    k_pair_probs<false><<<grid_for(n, 256, max_grid), 256, 0, s>>>(P, rule, r0, r, n, pe, pr);
+    paired ? go(k_pair_probs<true, true>) : go(k_pair_probs<true, false>);
 }
 
 void launch_propagate(const DevParams* P, int rule, const double* r0, const double* u, int64_t n, double* out,

@@ -139,11 +139,12 @@ void launch_init_positions(const StepLaunch& L, const int32_t* rep_of, const int
                            uint32_t n, cudaStream_t s);
 void launch_count(const StepLaunch& L, cudaStream_t s);
 void launch_pair_probs(const DevParams* P, int rule, const double* r0, const double* r, int64_t n, double* pe,
-                       double* pr, int max_grid, bool mixed3d, cudaStream_t s);
+                       double* pr, int max_grid, bool mixed3d, bool paired, cudaStream_t s);
 // kind 3 with fwd != nullptr: the 2D inverse table from the forward -ln(tail) table fwd
-// (quad2: the paired rows of Tab2::q2, or null)
-void launch_build_table(const DevParams* P, int rule, int kind, float* out, float4* quad, float4* quad2, int n0, int n1, double h,
+void launch_build_table(const DevParams* P, int rule, int kind, float* out, float4* quad, int n0, int n1, double h,
                         double h1, double* tot, const Tab2* fwd, int device_sms, cudaStream_t s);
+// the paired rows (Tab2::q2) of a finished table
+void launch_table_pairs(const float4* quad, int n0, int n1, float4* quad2, int device_sms, cudaStream_t s);
 // warp: one warp per draw (FP64 in 2D), else one thread
 void launch_resample(const DevParams* P, int rule, const double* r0, const double* u, int64_t n, double* out,
                      bool warp, int max_grid, cudaStream_t s);
