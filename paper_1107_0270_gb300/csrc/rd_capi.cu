@@ -56,6 +56,7 @@ struct rd_handle {
   double tuned_ms = 0.0;
   double factor = 1.0;               // cell-edge factor in use
   int reach = 1;                     // stencil reach of the cell sweep (2: 2D cells of half a cut-off)
+  int64_t max_cells = 0;             // cells that the cell arrays hold (the autotuner's largest grid)
   // staging of rd_set_state / rd_get_state (allocated on first use, capacity-sized)
   double* st_x = nullptr;
   int32_t* st_sp = nullptr;
@@ -123,6 +124,20 @@ static int device_sms() {
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
   cache[dev] = sms;
   return sms;
+}
+
+// The arrays that every completed step leaves as it found them: no cell holds a particle, no particle is
+// in a pair, no minimum offered, no consumed or new particle counted.
+static cudaError_t rest_arrays(rd_handle* h) {
+  const StepLaunch& L = h->L;
+  const size_t cap = (size_t)L.cap_particles, R = (size_t)h->cfg.n_replicas;
+  cudaError_t e = cudaMemsetAsync(L.cell_count, 0, (size_t)h->max_cells * 4, h->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(L.deg, 0, cap * 4, h->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(L.best_key, 0xFF, cap * 8, h->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(L.best_pid, 0xFF, cap * 8, h->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(L.rep_cons, 0, R * 4, h->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(L.rep_prod, 0, R * 4, h->stream);
+  return e;
 }
 
 static StepLaunch launch_for(rd_handle* h, int cur) {
@@ -633,6 +648,7 @@ static cudaError_t autotune(rd_handle* h) {
     cudaMemcpy(h->L.reps, cur.data(), rbytes, cudaMemcpyHostToDevice);
     cudaMemcpy(h->xbuf[0], sx, xbytes, cudaMemcpyDeviceToDevice);
     cudaMemcpy(h->idbuf[0], si, ibytes, cudaMemcpyDeviceToDevice);
+    if (now.status) rest_arrays(h);      // a trial step was aborted
     h->cur = 0;
   };
   auto trial = [&]() -> float {
@@ -924,15 +940,10 @@ int rd_init(const rd_config* cfg, void* stream, rd_handle** out) {
     delete h;
     return cuda_fail(e);
   };
-  cudaError_t e = cudaSuccess;
-  e = cudaMemsetAsync(L.cell_count, 0, max_cells * 4, h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(L.deg, 0, cap * 4, h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(L.best_key, 0xFF, cap * 8, h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(L.best_pid, 0xFF, cap * 8, h->stream);
+  h->max_cells = max_cells;
+  cudaError_t e = rest_arrays(h);
   if (e == cudaSuccess) e = cudaMemsetAsync(L.flags, 0, 2 * L.flag_stride * 4, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(L.status, 0, cap * 4, h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(L.rep_cons, 0, (size_t)c.n_replicas * 4, h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(L.rep_prod, 0, (size_t)c.n_replicas * 4, h->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync((void*)L.P, &h->hp, sizeof(DevParams), cudaMemcpyHostToDevice, h->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(L.reps, h->reps_init.data(), c.n_replicas * sizeof(RepDev), cudaMemcpyHostToDevice, h->stream);
@@ -1182,13 +1193,7 @@ int rd_set_state(rd_handle* h, int64_t n, const double* x, const int32_t* specie
   RD_CUDA(cudaStreamSynchronize(s));
   if (err & 1) return RD_EINVAL;
   h->cur = spare;
-  if (err) {
-    // the replaced state had an aborted step: the matching's arrays may not be at rest
-    const size_t cap = (size_t)h->L.cap_particles;
-    RD_CUDA(cudaMemsetAsync(h->L.deg, 0, cap * 4, s));
-    RD_CUDA(cudaMemsetAsync(h->L.best_key, 0xFF, cap * 8, s));
-    RD_CUDA(cudaMemsetAsync(h->L.best_pid, 0xFF, cap * 8, s));
-  }
+  if (err) RD_CUDA(rest_arrays(h));      // the replaced state had an aborted step
   // the counts of the new state follow in stream order (the next call that reads them synchronises)
   launch_count(launch_for(h, h->cur), s);
   RD_CUDA(cudaGetLastError());

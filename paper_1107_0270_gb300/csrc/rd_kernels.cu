@@ -3130,8 +3130,12 @@ __global__ void k_set_state_finish(const DevParams* __restrict__ Pp, RepDev* __r
   }
   if (threadIdx.x == 0) {
     if (ctl->status) {
-      *err = 2;                     // the host resets what an aborted step may have left behind
-      ctl->bar_count = ctl->bar2_count = 0u;
+      // what an aborted step may have left behind (a fused launch that gives up at a barrier does not reach
+      // its compaction, which puts the step's counters back); the host resets the arrays
+      *err = 2;
+      ctl->fired = ctl->n_conflict = ctl->n_decay = ctl->n_accept = ctl->n_round_acc = 0u;
+      ctl->n_ang = ctl->n_ev = ctl->done_blocks = ctl->done_res = 0u;
+      ctl->bar_count = ctl->bar2_count = ctl->live[0] = ctl->live[1] = 0u;
     }
     ctl->n = (uint32_t)n;
     ctl->step = (uint32_t)step;
