@@ -126,9 +126,10 @@ typedef struct {
                                          fused cooperative launch), 1 always fused, 2 always
                                          separate kernels.  Both give bit-identical results;
                                          RD_EINVAL outside 0..2 */
-  int32_t force_paths;                /* 0 normally.  Bit 0: conflict rounds on the whole cooperative
-                                         grid for any number of conflict pairs (normally only above
-                                         2048); bit 1: short conflict lists in global memory instead
+  int32_t force_paths;                /* 0 normally.  Bit 0: conflict rounds on three quarters of the
+                                         cooperative grid for any number of conflict pairs (normally
+                                         above 2048, on a block per 256 pairs up to that; all of it
+                                         in FP64 2D); bit 1: short conflict lists in global memory instead
                                          of shared memory.  For tests of the large-size code paths at
                                          small sizes; results are the same */
   int32_t angle_mode;                 /* direction of an encountered pair's new separation (Eq.

@@ -157,7 +157,7 @@ def make_config(system, precision: Optional[str] = None, capacity_factor: float 
     cell_reach: 0 automatic, 1 cells of a cut-off, 2 (2D) cells of half a cut-off, two-cell stencil.
     step_launch: "auto", "fused" (the whole step as one cooperative launch) or "separate" (one
     launch per kernel); both give bit-identical results.
-    force_paths: bit 0 conflict rounds on the whole grid at any size, bit 1 short conflict lists in
+    force_paths: bit 0 conflict rounds on most of the grid at any size, bit 1 short conflict lists in
     global memory (test knobs for the large-size paths; results unchanged)."""
     cfg = _Config()
     cfg.dim = int(system.dim)

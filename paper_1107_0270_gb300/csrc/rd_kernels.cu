@@ -1719,7 +1719,10 @@ __device__ __forceinline__ void ph_match_resolve(
   // no conflict pair, meanwhile.  (With the whole grid in the rounds and everything resolved after them,
   // 15 000 conflict pairs and 26 000 resolutions of a crowded 2D box took 82 us.)
   uint32_t nrb = nc > 0 && gridDim.x > 1 ? 1u : 0u;
-  if (multi) nrb = by_warp ? gridDim.x : min((nc + blockDim.x - 1) / blockDim.x, gridDim.x - gridDim.x / 4);
+  // (a test's limit of 0 pairs a block: the three quarters at any length)
+  const uint32_t most = gridDim.x - gridDim.x / 4;
+  if (multi)
+    nrb = by_warp ? gridDim.x : P.match_single_max == 0u ? most : min((nc + blockDim.x - 1) / blockDim.x, most);
   unsigned long long n_react = 0, n_res = 0, n_near = 0, n_rec = 0;
   if (blockIdx.x >= nrb) {
     const uint32_t nblk = gridDim.x - nrb, b = blockIdx.x - nrb;
