@@ -166,6 +166,7 @@ def algorithmic_bytes(kernel, precision, w):
     v = 16 if precision == "mixed" else 32
     n, nb, cells = w["n"], w["nb"], w["cells"]
     fired, acc, dec = w["fired"], w["accepted"], w["decays"]
+    consumed = dec + 2 * w.get("reactions", 0)
     table = {
         # read position + id; write end position, status, cell, slot; one cell counter per binned
         "k_prepare": n * (2 * v + 16) + 4 * nb,
@@ -182,8 +183,9 @@ def algorithmic_bytes(kernel, precision, w):
         # one 160-B job per resolved pair or decay pair left to it; write two positions (only
         # when directions come from the full propagator)
         "k_angles": (acc + dec) * (160 + 2 * v) if w.get("angles") else 0,
-        # read status, end position, id; write position + id (the scan stays on chip)
-        "k_compact": n * (2 * v + 12),
+        # read end position, id; write position + id; the consumed particles' list (8 bytes each, up to
+        # 4096), or every status word where there are more
+        "k_compact": n * (2 * v + 8) + (8 * consumed if consumed <= 4096 else 4 * n),
     }
     table["k_step_fused"] = sum(table.values())      # the whole step in one launch
     # the fused launch's two matching phases split the matching kernel's bytes
@@ -409,7 +411,8 @@ def run_ours(args, rank, world, local_rank):
         per = max(steps_done, 1)
         work = {"n": n_now, "nb": int(np.sum(np.isin(st["species"], [0, 1]))), "cells": layout["cells"],
                 "fired": d_stats["fired"] / per, "accepted": d_stats["matched"] / per,
-                "decays": d_stats["decays"] / per, "angles": args.angle == "exact"}
+                "decays": d_stats["decays"] / per, "reactions": d_stats["reactions"] / per,
+                "angles": args.angle == "exact"}
         cand_per_step = cand_local / per
         peak, peak_kind = measured_peaks()
         ab = algorithmic_bytes(dominant, args.precision, work)

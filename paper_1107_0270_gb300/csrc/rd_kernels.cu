@@ -1905,7 +1905,8 @@ __device__ __forceinline__ void ph_match_resolve(
 // The whole matching and resolution of a step with at most one block's threads of fired pairs and
 // decays, by one block: thread q takes pair q, or decay q - nf.  Pairs of degree 1 are accepted at once,
 // the rest go through the shared-memory rounds; then every accepted pair and decay is resolved in one
-// pass.  The chain has no grid barrier and no lists between its stages: 110 pairs 21 -> 14 us.
+// pass.  The chain has no grid barrier and no lists between its stages: 110 pairs and decays of the
+// 125 000-particle system 21.0 -> 18.4 us live.
 template <class T>
 __device__ __forceinline__ void match_resolve_few(
     const DevParams* Pp, DevCtl* ctl, const RepDev* reps, const FiredPair* fired, uint32_t* fstate, int32_t* matched,

@@ -77,7 +77,7 @@ static constexpr LapTab h_lap = make_lap_tab();
 //   u_{n-1} = n / (n - 1/2)^2 [2 (n + x) u_n - (n + 1) u_{n+1}],
 //   e^x K_0 = sqrt(pi / 2x) u_0 / sum u_n,  K_1 = K_0 (x + 1/2 - u_1 / u_0) / x,
 // started 12 + 280 / (|x| + Re x) orders up (both forms checked against 30-digit values: relative
-// error below 1e-14 for |x| in 0.3..60 and any phase in the right half plane).
+// error below 2e-14 for |x| in 0.3..60 and any phase in the right half plane).
 RD_HD void k01_scaled(cplx x, cplx& k0, cplx& k1) {
   const double ax = sqrt(x.re * x.re + x.im * x.im), key = ax + x.re;
   const cplx ix = crcp(x);
